@@ -422,12 +422,12 @@ mars_status mars_cache_set_state(mars_cache* cache, const mars_cache_state* stat
  *   current value in mars_cache_set_launch.
  * lane_min_pixels: the smallest image split over the lanes (default 2^17;
  *   at least 2); 0 keeps the current value.
- * Default: 128 threads, no cap, the occupancy maximum, every depth wave on the
+ * Default: 128 threads, the library's choice of cap, the occupancy maximum, every depth wave on the
  * same grid.  Errors: INVALID_ARG, CUDA. */
 typedef struct {
   int32_t threads[4];
   int32_t blocks_per_sm[4];
-  int32_t max_registers[4];  /* register cap of the compiled variant: 0 = the compiler's
+  int32_t max_registers[4];  /* register cap of the compiled variant: 0 = the library's
                                 choice; shade and reverse also 80 or 64, trace and shadow 64 or 40 */
   int32_t lanes;
   int32_t lane_min_pixels;
@@ -440,10 +440,11 @@ mars_status mars_cache_set_launch(mars_cache* cache, const mars_launch_config* c
  * by the kernel's device time over `repeats` (1..100) renders of `params`'s
  * iteration, rendered without statistics, guide deposits or image statistics
  * so that the cache's learned state is unchanged; keeps the fastest shape.
- * Then, for a cache with more than one lane and an image of at least 2^14
- * pixels, times whole iterations (as rendered outside profiling: graphs, lanes)
- * with one lane and with all lanes for any image of that size, and keeps the
- * faster.  Writes the result to `chosen` (may be NULL).  Synchronises `stream`
+ * Then times whole iterations (as rendered outside profiling: graphs, lanes)
+ * with the shape found and with the one the cache had, and, for a cache with
+ * more than one lane and an image of at least 2^14 pixels, each with one lane
+ * and with all lanes for any image of that size, and keeps the
+ * fastest.  Writes the result to `chosen` (may be NULL).  Synchronises `stream`
  * after every render.  Errors: INVALID_ARG, and those of mars_render_iteration. */
 mars_status mars_cache_autotune(mars_cache* cache, const mars_iter_params* params, int32_t repeats,
                                 mars_launch_config* chosen, void* stream);

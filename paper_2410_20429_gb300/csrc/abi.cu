@@ -1087,7 +1087,7 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
         const bool own = concurrent && l >= 1;
         cudaStream_t side2 = own ? (c->lane_side2.empty() ? nullptr : c->lane_side2[l - 1]) : c->side2;
         if ((r = launch_tile(s->ds, lane_cache(c, l), lane_arena(c, l, nl), c->d_args + t, c->launch,
-                             own ? c->lane_st[l - 1] : q, own ? c->lane_side[l - 1] : c->side, side2,
+                             tiles[t].second - tiles[t].first, own ? c->lane_st[l - 1] : q, own ? c->lane_side[l - 1] : c->side, side2,
                              own ? c->lane_sync[l - 1].data() : c->sync_events.data(), ev)) != cudaSuccess)
           return r;
       }
@@ -1682,10 +1682,14 @@ mars_status mars_cache_autotune(mars_cache* c, const mars_iter_params* params, i
   p.combine = 0;
   p.profile = 1;
   int threads[WAVE_KERNELS], bps[WAVE_KERNELS], var[WAVE_KERNELS];
+  int threads0[WAVE_KERNELS], bps0[WAVE_KERNELS], var0[WAVE_KERNELS];
   for (int k = 0; k < WAVE_KERNELS; ++k) {
     threads[k] = c->launch.threads[k];
     bps[k] = c->blocks_per_sm[k];
     var[k] = c->launch.variant[k];
+    threads0[k] = threads[k];
+    bps0[k] = bps[k];
+    var0[k] = var[k];
   }
   auto time_of = [&](int k, double* ms) -> mars_status {
     mars_status rc = apply_launch(c, threads, bps, var);
@@ -1707,6 +1711,7 @@ mars_status mars_cache_autotune(mars_cache* c, const mars_iter_params* params, i
     int best_t = threads[k], best_b = bps[k], best_v = var[k];
     double best = 1e300;
     for (int v = 0; v < wave_variants(k); ++v) {
+      if (wave_variant_repeats(k, v)) continue;
       for (int ti = 0; ti < 3; ++ti) {
         int occ[WAVE_KERNELS];
         int tt[WAVE_KERNELS] = {threads[0], threads[1], threads[2], threads[3]};
@@ -1737,48 +1742,61 @@ mars_status mars_cache_autotune(mars_cache* c, const mars_iter_params* params, i
     bps[k] = best_b;
     var[k] = best_v;
   }
-  mars_status rc = apply_launch(c, threads, bps, var);
-  if (rc != MARS_OK) return rc;
-  // Tile lanes: whole iterations as rendered outside profiling (graph replay,
-  // concurrent lanes), one lane against all of them, timed on the stream.
-  if (c->lanes > 1 && c->pixels >= kLaneFloorPixels) {
-    mars_iter_params q = p;
-    q.profile = 0;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
-      if (e0) cudaEventDestroy(e0);
-      return set_error(MARS_ERR_CUDA, "event create failed");
-    }
-    const int cand_lanes[2] = {1, c->lanes};
-    const int64_t cand_min[2] = {c->lane_min_pixels,
-                                 std::max<int64_t>(kLaneFloorPixels, std::min<int64_t>(kLaneMinPixels, c->pixels))};
-    double best = 1e300;
-    int best_k = 0;
-    for (int k = 0; k < 2 && rc == MARS_OK; ++k) {
-      c->use_lanes = cand_lanes[k];
-      c->lane_min_pixels = cand_min[k];
-      double tot = 0.0;
-      for (int r = 0; r <= repeats && rc == MARS_OK; ++r) {  // the first render warms up (and records the graph)
-        mars_iter_stats st{};
-        float ms = 0.f;
-        if (cudaEventRecord(e0, (cudaStream_t)stream) != cudaSuccess) rc = set_error(MARS_ERR_CUDA, "event record");
-        if (rc == MARS_OK) rc = render_iteration_impl(c, &q, nullptr, &st, (cudaStream_t)stream);
-        if (rc == MARS_OK && (cudaEventRecord(e1, (cudaStream_t)stream) != cudaSuccess ||
-                              cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
-          rc = set_error(MARS_ERR_CUDA, "event timing");
-        if (r > 0) tot += ms;
-      }
-      if (rc == MARS_OK && tot < best) {
-        best = tot;
-        best_k = k;
-      }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (rc != MARS_OK) return rc;
-    c->use_lanes = cand_lanes[best_k];
-    c->lane_min_pixels = cand_min[best_k];
+  // Whole iterations as rendered outside profiling (graph replay, concurrent
+  // streams and lanes), timed on the stream: the shape found above against the
+  // one the cache came with -- a kernel timed alone does not show what its shape
+  // leaves to the kernels beside it -- each with one lane and, where the image
+  // is large enough, with all of them.
+  const int64_t tuned_min = std::max<int64_t>(kLaneFloorPixels, std::min<int64_t>(kLaneMinPixels, c->pixels));
+  const bool try_lanes = c->lanes > 1 && c->pixels >= kLaneFloorPixels;
+  mars_iter_params q = p;
+  q.profile = 0;
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
+    if (e0) cudaEventDestroy(e0);
+    return set_error(MARS_ERR_CUDA, "event create failed");
   }
+  const int64_t min0 = c->lane_min_pixels;
+  const int lanes0 = c->use_lanes;
+  mars_status rc = MARS_OK;
+  auto use = [&](int k) -> mars_status {  // bit 0: all lanes, bit 1: the tuned shape
+    if (try_lanes) {
+      c->use_lanes = (k & 1) ? c->lanes : 1;
+      c->lane_min_pixels = (k & 1) ? tuned_min : min0;
+    }
+    return (k & 2) ? apply_launch(c, threads, bps, var) : apply_launch(c, threads0, bps0, var0);
+  };
+  double best = 1e300;
+  int best_k = -1;
+  for (int k = 0; k < 4 && rc == MARS_OK; ++k) {
+    if ((k & 1) && !try_lanes) continue;
+    rc = use(k);
+    double tot = 0.0;
+    for (int r = 0; r <= 2 * repeats && rc == MARS_OK; ++r) {  // the first render warms up (and records the graph)
+      mars_iter_stats st{};
+      float ms = 0.f;
+      if (cudaEventRecord(e0, (cudaStream_t)stream) != cudaSuccess) rc = set_error(MARS_ERR_CUDA, "event record");
+      if (rc == MARS_OK) rc = render_iteration_impl(c, &q, nullptr, &st, (cudaStream_t)stream);
+      if (rc == MARS_OK && (cudaEventRecord(e1, (cudaStream_t)stream) != cudaSuccess ||
+                            cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+        rc = set_error(MARS_ERR_CUDA, "event timing");
+      if (r > 0) tot += ms;
+    }
+    if (rc == MARS_OK && tot < best) {
+      best = tot;
+      best_k = k;
+    }
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (best_k < 0) {
+    c->use_lanes = lanes0;
+    c->lane_min_pixels = min0;
+    return rc;
+  }
+  const mars_status rk = use(best_k);
+  if (rc == MARS_OK) rc = rk;
+  if (rc != MARS_OK) return rc;
   if (chosen) return mars_cache_get_launch(c, chosen);
   return MARS_OK;
 }

@@ -275,7 +275,7 @@ int light_variants();
 // side2: the light connection kernels' stream (light connections only; null:
 // they run on side); sync: D + 2 events
 cudaError_t launch_tile(const DevScene& s, const DevCache& c, const Arena& a, const IterArgs* it,
-                        const WaveLaunch& L, cudaStream_t st, cudaStream_t side, cudaStream_t side2,
+                        const WaveLaunch& L, int64_t tile_pixels, cudaStream_t st, cudaStream_t side, cudaStream_t side2,
                         const cudaEvent_t* sync, cudaEvent_t* ev);
 // adds a second tile lane's iteration totals into the first lane's counters
 cudaError_t launch_merge_lanes(DevCounters* dst, DevCounters* src, cudaStream_t st);
@@ -283,7 +283,8 @@ cudaError_t launch_merge_lanes(DevCounters* dst, DevCounters* src, cudaStream_t 
 cudaError_t wave_occupancy(const int threads[WAVE_KERNELS], const int variant[WAVE_KERNELS],
                            int blocks_per_sm[WAVE_KERNELS]);
 int wave_variants(int kernel);                    // compiled register-cap variants of a wave kernel
-int wave_variant_registers(int kernel, int v);    // its register cap (0: the compiler's choice)
+int wave_variant_registers(int kernel, int v);    // its register cap (0: the library's choice)
+bool wave_variant_repeats(int kernel, int v);     // the same code as variant 0
 bool wave_threads_ok(int threads);
 int tile_launches(int max_depth, int techniques);  // kernels launch_tile issues
 // image statistics (stats.cu)

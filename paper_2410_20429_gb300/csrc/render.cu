@@ -24,6 +24,8 @@
 //                      cells in a warp before float64 atomics.
 //
 // A tile whose arena overflowed commits nothing.
+#include <algorithm>
+
 #include "device.cuh"
 
 namespace mars {
@@ -1075,18 +1077,24 @@ __global__ void __launch_bounds__(MAX_WAVE_THREADS, MINB) k_reverse(const DevSce
 
 size_t shade_smem(int threads) { return (size_t)(threads / 32) * sizeof(ShadeWarpCtx); }
 
-// Register-cap variants of every wave kernel: variant v is compiled with
-// __launch_bounds__(256, MINB) for MINB = 1 (the compiler's choice), or a cap
-// that lets more blocks share an SM (shade and reverse: 80 and 64 registers;
-// trace and shadow: 64 and 40 registers), trading spills for occupancy.
+// Register-cap variants of every wave kernel, compiled with
+// __launch_bounds__(256, MINB): trace and shadow 64 or 40 registers, shade 80 or
+// 64, reverse the compiler's choice (110), 80 or 64.  Variant 0, what a cache
+// starts with, is the 64, 80 and 64 register one for trace, shade and shadow:
+// uncapped they take 88, 144 and 77, and the kernels, which wait on loads most of
+// the time, lose more to the warps that then do not fit than they gain
+// (iterations with the caps against without: guided room 512^2 0.94 -> 0.89 ms
+// in the warm-up and 1.44 -> 1.25 with learned counts, 131k triangles at 1024^2
+// 3.62 -> 2.97, 524k at 2048^2 13.4 -> 11.7).  k_reverse keeps its registers
+// (capped at 80, 512^2 warm-up 0.86 -> 0.91 ms).
 using TraceFn = void (*)(const DevScene, const DevCache, const Arena, const IterArgs*, const int);
 using ShadowFn = void (*)(const DevScene, const DevCache, const Arena, const int);
-TraceFn trace_fn(int v) { return v == 2 ? k_trace<6> : (v == 1 ? k_trace<4> : k_trace<1>); }
+TraceFn trace_fn(int v) { return v == 2 ? k_trace<6> : k_trace<4>; }
 TraceFn shade_fn(int v, bool bd = false) {
-  if (bd) return v == 2 ? k_shade<4, true> : (v == 1 ? k_shade<3, true> : k_shade<1, true>);
-  return v == 2 ? k_shade<4, false> : (v == 1 ? k_shade<3, false> : k_shade<1, false>);
+  if (bd) return v == 2 ? k_shade<4, true> : k_shade<3, true>;
+  return v == 2 ? k_shade<4, false> : k_shade<3, false>;
 }
-ShadowFn shadow_fn(int v) { return v == 2 ? k_shadow<6> : (v == 1 ? k_shadow<4> : k_shadow<1>); }
+ShadowFn shadow_fn(int v) { return v == 2 ? k_shadow<6> : k_shadow<4>; }
 TraceFn reverse_fn(int v, bool bd = false) {
   if (bd) return v == 2 ? k_reverse<4, true> : (v == 1 ? k_reverse<3, true> : k_reverse<1, true>);
   return v == 2 ? k_reverse<4, false> : (v == 1 ? k_reverse<3, false> : k_reverse<1, false>);
@@ -1095,6 +1103,7 @@ TraceFn reverse_fn(int v, bool bd = false) {
 }  // namespace
 
 int wave_variants(int) { return 3; }
+bool wave_variant_repeats(int kernel, int v) { return v == 1 && kernel != WK_REVERSE; }
 int wave_variant_registers(int kernel, int v) {
   if (v == 0) return 0;
   if (kernel == WK_SHADE || kernel == WK_REVERSE) return v == 1 ? 80 : 64;
@@ -1121,12 +1130,19 @@ cudaError_t wave_occupancy(const int threads[WAVE_KERNELS], const int variant[WA
 bool wave_threads_ok(int threads) { return threads >= 32 && threads <= MAX_WAVE_THREADS && threads % 32 == 0; }
 
 cudaError_t launch_tile(const DevScene& s, const DevCache& c, const Arena& a, const IterArgs* it, const WaveLaunch& L,
-                        cudaStream_t st, cudaStream_t side, cudaStream_t side2, const cudaEvent_t* sync,
+                        int64_t tile_pixels, cudaStream_t st, cudaStream_t side, cudaStream_t side2, const cudaEvent_t* sync,
                         cudaEvent_t* ev) {
   k_tile_init<<<1, 32, 0, st>>>(c.ctr, it);
   const int D = c.max_depth;
   const int tT = L.threads[WK_TRACE], tS = L.threads[WK_SHADE], tH = L.threads[WK_SHADOW], tR = L.threads[WK_REVERSE];
-  auto G = [&](int k, int) { return L.grid[k]; };
+  // The persistent grid, but no more blocks than four rays per pixel of the
+  // tile fill: a block without work still costs its launch (64^2 box 0.150 ->
+  // 0.147 ms, 128^2 room 0.605 -> 0.596 ms; two rays per pixel 0.617, one 0.667:
+  // the second and third waves hold more rays than there are pixels)
+  auto G = [&](int k, int) {
+    const int64_t most = (4 * tile_pixels + L.threads[k] - 1) / L.threads[k];
+    return (int)std::max<int64_t>(1, std::min<int64_t>(L.grid[k], most));
+  };
   const size_t smS = shade_smem(tS);
   const bool nee = (c.techniques & MARS_TECH_NEE) != 0;
   const bool bd = (c.techniques & MARS_TECH_LIGHT) != 0;
