@@ -347,40 +347,39 @@ mars_status scene_create_impl(const mars_scene_desc* d, cudaStream_t st, mars_sc
   };
   cudaError_t e;
   if ((e = dev_alloc((void**)&s->d_prims, sizeof(float4) * prims.size(), st)) != cudaSuccess) return cleanup(e, "scene alloc");
-  if ((e = dev_alloc((void**)&s->d_boxes, sizeof(float4) * boxes.size(), st)) != cudaSuccess) return cleanup(e, "scene alloc");
-  if ((e = dev_alloc((void**)&s->d_nodes, sizeof(BvhNode) * std::max(1, n - 1), st)) != cudaSuccess) return cleanup(e, "scene alloc");
   if ((e = dev_alloc((void**)&s->d_mats, sizeof(float4) * mats.size(), st)) != cudaSuccess) return cleanup(e, "scene alloc");
   if ((e = dev_alloc((void**)&s->d_lights, sizeof(float4) * lights.size(), st)) != cudaSuccess) return cleanup(e, "scene alloc");
   if ((e = cudaMemcpyAsync(s->d_prims, prims.data(), sizeof(float4) * prims.size(), cudaMemcpyHostToDevice, st)) ||
-      (e = cudaMemcpyAsync(s->d_boxes, boxes.data(), sizeof(float4) * boxes.size(), cudaMemcpyHostToDevice, st)) ||
       (e = cudaMemcpyAsync(s->d_mats, mats.data(), sizeof(float4) * mats.size(), cudaMemcpyHostToDevice, st)) ||
       (e = cudaMemcpyAsync(s->d_lights, lights.data(), sizeof(float4) * lights.size(), cudaMemcpyHostToDevice, st)))
     return cleanup(e, "scene upload");
   NvtxRange nvtx_bvh("mars:bvh_build");
+  // the binary hierarchy, on the host: built there (SAH), or read back (LBVH)
+  std::vector<BvhNode> bin(std::max(0, n - 1));
   if (d->bvh == MARS_BVH_SAH && n >= 2) {
-    std::vector<BvhNode> sah;
-    if (!build_bvh_sah(boxes, n, sah)) {
+    if (!build_bvh_sah(boxes, n, bin)) {
       set_error(MARS_ERR_CUDA, "SAH build produced an invalid hierarchy");
       scene_destroy_impl(s);
       return MARS_ERR_CUDA;
     }
-    if ((e = cudaMemcpyAsync(s->d_nodes, sah.data(), sizeof(BvhNode) * (n - 1), cudaMemcpyHostToDevice, st)) !=
-        cudaSuccess)
-      return cleanup(e, "BVH upload");
-  } else {
+  } else if (n >= 2) {
     std::string berr;
-    if ((e = build_bvh(s->d_boxes, n, s->ds.lo, s->ds.ext, s->d_nodes, st, &berr)) != cudaSuccess)
-      return cleanup(e, berr.c_str());
+    float4* d_boxes = nullptr;
+    BvhNode* d_bin = nullptr;
+    if ((e = dev_alloc((void**)&d_boxes, sizeof(float4) * boxes.size(), st)) == cudaSuccess &&
+        (e = dev_alloc((void**)&d_bin, sizeof(BvhNode) * (n - 1), st)) == cudaSuccess &&
+        (e = cudaMemcpyAsync(d_boxes, boxes.data(), sizeof(float4) * boxes.size(), cudaMemcpyHostToDevice, st)) ==
+            cudaSuccess &&
+        (e = build_bvh(d_boxes, n, s->ds.lo, s->ds.ext, d_bin, st, &berr)) == cudaSuccess)
+      e = cudaMemcpyAsync(bin.data(), d_bin, sizeof(BvhNode) * (n - 1), cudaMemcpyDeviceToHost, st);
+    dev_free(d_boxes, st);
+    dev_free(d_bin, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cleanup(e, berr.empty() ? "BVH build" : berr.c_str());
   }
-  if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cleanup(e, "scene create");
+  // check the hierarchy before any kernel traverses it: every internal node
+  // reached once from the root, every primitive once, all indices in range
   if (n >= 2) {
-    // check the hierarchy before any kernel traverses it: every internal node
-    // reached once from the root, every primitive once, all indices in range
-    std::vector<BvhNode> nodes(n - 1);
-    if ((e = cudaMemcpyAsync(nodes.data(), s->d_nodes, sizeof(BvhNode) * (n - 1), cudaMemcpyDeviceToHost, st)) !=
-            cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
-      return cleanup(e, "BVH readback");
     std::vector<uint8_t> seen_node(n - 1, 0), seen_leaf(n, 0);
     std::vector<int> stack{0};
     bool okb = true;
@@ -390,8 +389,8 @@ mars_status scene_create_impl(const mars_scene_desc* d, cudaStream_t st, mars_sc
       if (k < 0 || k >= n - 1 || seen_node[k]) { okb = false; break; }
       seen_node[k] = 1;
       int ch[2];
-      std::memcpy(&ch[0], &nodes[k].a.w, sizeof(int));
-      std::memcpy(&ch[1], &nodes[k].b.w, sizeof(int));
+      std::memcpy(&ch[0], &bin[k].a.w, sizeof(int));
+      std::memcpy(&ch[1], &bin[k].b.w, sizeof(int));
       for (int c : ch) {
         if (c < 0) {
           const int leaf = ~c;
@@ -410,95 +409,25 @@ mars_status scene_create_impl(const mars_scene_desc* d, cudaStream_t st, mars_sc
       return MARS_ERR_CUDA;
     }
   }
-  if (n >= 2) {
-    // collapse the binary hierarchy into 4-wide nodes: a node's children are
-    // grown by replacing the internal child with the largest box surface by its
-    // two children until there are four or only leaves remain
-    std::vector<BvhNode> bin(n - 1);
-    if ((e = cudaMemcpyAsync(bin.data(), s->d_nodes, sizeof(BvhNode) * (n - 1), cudaMemcpyDeviceToHost, st)) !=
-            cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
-      return cleanup(e, "BVH readback");
-    struct Ch {
-      int id;              // >= 0 binary internal node, < 0 ~primitive
-      float lo[3], hi[3];
-    };
-    auto kids = [&](int k, Ch out[2]) {
-      const BvhNode& b = bin[k];
-      int l, r;
-      std::memcpy(&l, &b.a.w, sizeof(int));
-      std::memcpy(&r, &b.b.w, sizeof(int));
-      out[0] = {l, {b.a.x, b.a.y, b.a.z}, {b.b.x, b.b.y, b.b.z}};
-      out[1] = {r, {b.c.x, b.c.y, b.c.z}, {b.d.x, b.d.y, b.d.z}};
-    };
-    auto area = [](const Ch& c) {
-      const double dx = c.hi[0] - c.lo[0], dy = c.hi[1] - c.lo[1], dz = c.hi[2] - c.lo[2];
-      return dx * dy + dy * dz + dz * dx;
-    };
-    std::vector<Bvh4Node> n4;
-    n4.reserve(n);
-    std::vector<std::pair<int, int>> todo;  // (binary node, BVH4 slot)
-    n4.emplace_back();
-    todo.emplace_back(0, 0);
-    while (!todo.empty()) {
-      const auto [bk, slot] = todo.back();
-      todo.pop_back();
-      Ch set[4];
-      int m = 2;
-      kids(bk, set);
-      while (m < 4) {
-        int best = -1;
-        double ba = -1.0;
-        for (int k = 0; k < m; ++k)
-          if (set[k].id >= 0 && area(set[k]) > ba) { ba = area(set[k]); best = k; }
-        if (best < 0) break;
-        Ch two[2];
-        kids(set[best].id, two);
-        set[best] = two[0];
-        set[m++] = two[1];
-      }
-      float lo[3][4], hi[3][4];
-      int ch[4];
-      for (int k = 0; k < 4; ++k) {
-        for (int a = 0; a < 3; ++a) {
-          lo[a][k] = k < m ? set[k].lo[a] : 0.0f;   // empty slot (child BVH4_EMPTY): never visited
-          hi[a][k] = k < m ? set[k].hi[a] : 0.0f;
-        }
-        if (k >= m) {
-          ch[k] = BVH4_EMPTY;
-        } else if (set[k].id < 0) {
-          ch[k] = set[k].id;
-        } else {
-          ch[k] = (int)n4.size();
-          n4.emplace_back();
-          todo.emplace_back(set[k].id, ch[k]);
-        }
-      }
-      Bvh4Node& nd = n4[slot];
-      nd.lox = make_float4(lo[0][0], lo[0][1], lo[0][2], lo[0][3]);
-      nd.loy = make_float4(lo[1][0], lo[1][1], lo[1][2], lo[1][3]);
-      nd.loz = make_float4(lo[2][0], lo[2][1], lo[2][2], lo[2][3]);
-      nd.hix = make_float4(hi[0][0], hi[0][1], hi[0][2], hi[0][3]);
-      nd.hiy = make_float4(hi[1][0], hi[1][1], hi[1][2], hi[1][3]);
-      nd.hiz = make_float4(hi[2][0], hi[2][1], hi[2][2], hi[2][3]);
-      nd.child = make_int4(ch[0], ch[1], ch[2], ch[3]);
-      nd.pad = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    if ((e = dev_alloc((void**)&s->d_nodes4, sizeof(Bvh4Node) * n4.size(), st)) != cudaSuccess)
-      return cleanup(e, "scene alloc");
-    if ((e = cudaMemcpyAsync(s->d_nodes4, n4.data(), sizeof(Bvh4Node) * n4.size(), cudaMemcpyHostToDevice, st)) !=
-            cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
-      return cleanup(e, "BVH4 upload");
-    s->ds.n_nodes4 = (int)n4.size();
+  std::vector<Bvh4Node> n4;
+  int entries = 0;
+  if (!collapse_bvh4(bin, boxes, n, n4, &entries)) {
+    set_error(MARS_ERR_CUDA, "the hierarchy needs %d traversal stack entries, more than %d", entries, TRAVERSAL_STACK);
+    scene_destroy_impl(s);
+    return MARS_ERR_CUDA;
   }
+  if ((e = dev_alloc((void**)&s->d_nodes4, sizeof(Bvh4Node) * n4.size(), st)) != cudaSuccess)
+    return cleanup(e, "scene alloc");
+  if ((e = cudaMemcpyAsync(s->d_nodes4, n4.data(), sizeof(Bvh4Node) * n4.size(), cudaMemcpyHostToDevice, st)) !=
+          cudaSuccess ||
+      (e = cudaStreamSynchronize(st)) != cudaSuccess)
+    return cleanup(e, "scene create");
+  s->ds.n_nodes4 = (int)n4.size();
   s->ds.nodes4 = s->d_nodes4;
   s->ds.prims = s->d_prims;
-  s->ds.nodes = s->d_nodes;
   s->ds.mats = s->d_mats;
   s->ds.lights = s->d_lights;
-  s->device_bytes = sizeof(float4) * (prims.size() + boxes.size() + mats.size() + lights.size()) +
-                    sizeof(BvhNode) * std::max(1, n - 1);
+  s->device_bytes = sizeof(float4) * (prims.size() + mats.size() + lights.size()) + sizeof(Bvh4Node) * n4.size();
   *out = s;
   return MARS_OK;
 }
@@ -511,8 +440,6 @@ void scene_destroy_impl(mars_scene* s) {
   cudaStream_t st = s->stream;
   if (cudaStreamQuery(st) == cudaErrorInvalidResourceHandle) st = cudaStreamPerThread;
   dev_free(s->d_prims, st);
-  dev_free(s->d_boxes, st);
-  dev_free(s->d_nodes, st);
   dev_free(s->d_nodes4, st);
   dev_free(s->d_mats, st);
   dev_free(s->d_lights, st);
@@ -624,8 +551,6 @@ mars_status cache_create_impl(const mars_scene* s, const mars_cache_desc* d, cud
   for (int k = 0; k < NSH; ++k)
     if ((e = dev_alloc((void**)&c->arena.SH[k], sizeof(float4) * c->arena.scap, st)) != cudaSuccess)
       return cleanup(e, "arena alloc");
-  if ((e = dev_alloc((void**)&c->arena.SL, sizeof(unsigned int) * c->arena.scap, st)) != cudaSuccess)
-    return cleanup(e, "arena alloc");
   if (c->arena.lcap) {
     if ((e = dev_alloc((void**)&c->arena.R5, sizeof(float4) * cap, st)) != cudaSuccess) return cleanup(e, "arena alloc");
     for (int k = 0; k < NLJ; ++k)
@@ -867,7 +792,6 @@ void cache_destroy_impl(mars_cache* c) {
   dev_free(c->arena.M, st);
   dev_free(c->arena.H, st);
   for (auto* p : c->arena.SH) dev_free(p, st);
-  dev_free(c->arena.SL, st);
   dev_free(c->arena.R5, st);
   for (auto* p : c->arena.LJ) dev_free(p, st);
   dev_free(c->arena.LR, st);
@@ -923,7 +847,6 @@ static Arena lane_arena(const mars_cache* c, int l, int nl) {
   a.M += r0;
   a.H += r0;
   for (auto& p : a.SH) p += s0;
-  a.SL += s0;
   if (a.lcap) {
     a.R5 += r0;
     for (auto& p : a.LJ) p += l0;

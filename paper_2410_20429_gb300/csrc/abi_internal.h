@@ -89,8 +89,6 @@ struct mars_scene {
   int width = 0, height = 0, n_prims = 0, n_lights = 0;
   mars::DevScene ds{};
   float4* d_prims = nullptr;
-  float4* d_boxes = nullptr;
-  mars::BvhNode* d_nodes = nullptr;
   mars::Bvh4Node* d_nodes4 = nullptr;
   float4* d_mats = nullptr;
   float4* d_lights = nullptr;

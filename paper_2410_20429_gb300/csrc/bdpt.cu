@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(MAX_LIGHT_THREADS, MINB) k_light_connect(const
       const float den = ta + tb + tc;
       const float wgt = den > 0.0f ? ta / den : 0.0f;
       ++n_conn;
-      if (!trace_any4(s, xo, w, dist - s.eps, tw)) val = C * wgt;
+      if (!trace_any(s, xo, w, dist - s.eps, tw)) val = C * wgt;
     }
     a.LC[vs] = f4(val, 0.0f);
   }

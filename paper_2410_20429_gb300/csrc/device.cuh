@@ -158,180 +158,227 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return r;
 }
 
-// slab test of one box against [0, tmax]; returns the entry distance, or NaN
-// on a miss (so that every comparison with it is false)
-__device__ __forceinline__ float box_entry(float4 lo, float4 hi, f3 o, f3 inv, float tmax) {
-  const float x0 = (lo.x - o.x) * inv.x, x1 = (hi.x - o.x) * inv.x;
-  const float y0 = (lo.y - o.y) * inv.y, y1 = (hi.y - o.y) * inv.y;
-  const float z0 = (lo.z - o.z) * inv.z, z1 = (hi.z - o.z) * inv.z;
-  const float tn = fmax3(fminf(x0, x1), fminf(y0, y1), fmaxf(fminf(z0, z1), 0.0f));
-  const float tf = fmin3(fmaxf(x0, x1), fmaxf(y0, y1), fminf(fmaxf(z0, z1), tmax));
-  return tn <= tf * 1.00000024f ? tn : __int_as_float(0x7fffffff);
+constexpr int STACK = TRAVERSAL_STACK;
+
+// A ray prepared for the slab tests of the 4-wide nodes.  A plane at coordinate
+// p is met at t = p / d - o / d: with o / d formed once per ray, one fused
+// multiply-add per plane instead of a subtraction and a product, and with the
+// nearer plane of each axis known from the sign of d no minimum or maximum
+// between an axis's two planes.  o / d is rounded, so the near constant is
+// lowered and the far one raised by 2^-22 of it (four times its rounding
+// error): a box is never left out that exact arithmetic would admit.  A component
+// of d that is zero (or below 1e-20, or not finite) counts as 1e-20: its planes
+// lie at huge distances on the side that tells whether the origin is between
+// them, as the infinities of a division by zero would, without their NaN.  An
+// origin that is not a number meets no box.
+struct SlabRay {
+  float ix, iy, iz;           // 1 / d
+  float nx, ny, nz;           // near plane constants
+  float fx, fy, fz;           // far plane constants
+  int kx, ky, kz;             // float4 of a node that holds the near planes of each axis
+};
+__device__ __forceinline__ SlabRay slab_ray(f3 o, f3 d) {
+  SlabRay r;
+  constexpr float TINY = 1e-20f, BIG = 1e20f;
+  r.ix = 1.0f / (fabsf(d.x) > TINY && fabsf(d.x) < BIG ? d.x : TINY);
+  r.iy = 1.0f / (fabsf(d.y) > TINY && fabsf(d.y) < BIG ? d.y : TINY);
+  r.iz = 1.0f / (fabsf(d.z) > TINY && fabsf(d.z) < BIG ? d.z : TINY);
+  const float ox = o.x * r.ix, oy = o.y * r.iy, oz = o.z * r.iz;
+  constexpr float SLACK = 2.3841858e-7f;   // 2^-22
+  const float ex = SLACK * fabsf(ox), ey = SLACK * fabsf(oy), ez = SLACK * fabsf(oz);
+  const float inf = __int_as_float(0x7f800000);
+  r.nx = ox == ox ? -ox - ex : inf; r.ny = oy == oy ? -oy - ey : inf; r.nz = oz == oz ? -oz - ez : inf;
+  r.fx = ex - ox; r.fy = ey - oy; r.fz = ez - oz;
+  r.kx = r.ix < 0.0f ? 3 : 0; r.ky = r.iy < 0.0f ? 4 : 1; r.kz = r.iz < 0.0f ? 5 : 2;
+  return r;
 }
 
-constexpr int STACK = 48;
-
-// Closest hit by stack traversal of the LBVH.  Ties in t go to the lower
-// primitive index, as in a brute-force scan in index order.
-__device__ __forceinline__ int trace_closest(const DevScene& s, f3 o, f3 d, float& t_best, TraceWork& w) {
-  t_best = __int_as_float(0x7f800000);
-  int best = -1;
-  if (s.n_prims == 1) {
-    float t;
-    if (hit_prim(s.prims, 0, o, d, t_best, t, w)) { t_best = t; best = 0; }
-    return best;
-  }
-  const f3 inv = mk3(1.0f / d.x, 1.0f / d.y, 1.0f / d.z);
-  int stack[STACK];
-  int sp = 0;
-  int node = 0;
-  // every internal node is visited at most once per ray
-  for (int visits = 0; visits < s.n_prims; ++visits) {
-    if (!trav_ok(node >= 0 && node < s.n_prims - 1, MARS_CHECK_NODE, w)) break;
-    const BvhNode nd = s.nodes[node];
-    ++w.nodes;
-    // admit boxes entered at t <= t_best (a tie may still win on index)
-    const float tl = box_entry(nd.a, nd.b, o, inv, t_best);
-    const float tr = box_entry(nd.c, nd.d, o, inv, t_best);
-    int cl = __float_as_int(nd.a.w), cr = __float_as_int(nd.b.w);
-    bool vl = tl <= t_best, vr = tr <= t_best;
-    // the admitted leaf children (left first) go through one copy of the
-    // primitive test, so that lanes with a leaf on either side share it
-    int p0 = -1, p1 = -1;
-    if (vl && cl < 0) {
-      p0 = ~cl;
-      vl = false;
-    }
-    if (vr && cr < 0) {
-      if (p0 < 0) p0 = ~cr; else p1 = ~cr;
-      vr = false;
-    }
-    while (p0 >= 0) {
-      if (!trav_ok(p0 < s.n_prims, MARS_CHECK_PRIM, w)) break;
-      float t;
-      if (hit_prim(s.prims, p0, o, d, t_best * 1.0000002f + 1e-30f, t, w) &&
-          (t < t_best || (t == t_best && p0 < best))) { t_best = t; best = p0; }
-      p0 = p1;
-      p1 = -1;
-    }
-    if (vl && vr) {
-      const bool lfirst = tl <= tr;
-      const int near = lfirst ? cl : cr, far = lfirst ? cr : cl;
-      if (sp < STACK) stack[sp++] = far;
-      node = near;
-    } else if (vl) {
-      node = cl;
-    } else if (vr) {
-      node = cr;
-    } else {
-      if (sp == 0) break;
-      node = stack[--sp];
-    }
-  }
-  return best;
-}
-
-// Entry distances of the four child boxes of a 4-wide node against [0, tmax]
-// (NaN for a miss or an empty slot), by the same slab arithmetic as box_entry.
-__device__ __forceinline__ void box4_entry(const Bvh4Node& nd, f3 o, f3 inv, float tmax, float t[4]) {
-  const float lx[4] = {nd.lox.x, nd.lox.y, nd.lox.z, nd.lox.w}, ly[4] = {nd.loy.x, nd.loy.y, nd.loy.z, nd.loy.w};
-  const float lz[4] = {nd.loz.x, nd.loz.y, nd.loz.z, nd.loz.w}, hx[4] = {nd.hix.x, nd.hix.y, nd.hix.z, nd.hix.w};
-  const float hy[4] = {nd.hiy.x, nd.hiy.y, nd.hiy.z, nd.hiy.w}, hz[4] = {nd.hiz.x, nd.hiz.y, nd.hiz.z, nd.hiz.w};
-  const int ch[4] = {nd.child.x, nd.child.y, nd.child.z, nd.child.w};
+// Entry distances t of the four child boxes of a node and the exits of their
+// overlap with [0, tmax]: child k is met if t[k] <= e[k].  The unused slots of a
+// node hold an inverted infinite box, which no ray meets.  Returns the children.
+// The float4 j of node n is stored at place j ^ (n & 7) of the node's eight: the
+// lanes of a warp read the same j of different nodes, which at one place of
+// 128-byte nodes would all lie in the same four shared-memory banks of the L1
+// cache (guided room 512^2, first bounce: 48 -> 33 % of the L1's data-stage
+// cycles, 131 -> 122 us).
+__device__ __forceinline__ int4 box4(const float4* __restrict__ nodes, int node, const SlabRay& r, float tmax, float t[4],
+                                     float e[4]) {
+  const float4* nd = nodes + 8u * (unsigned)node;
+  const int z = node & 7;
+  const float4 nx = __ldg(nd + (r.kx ^ z)), fx = __ldg(nd + ((3 - r.kx) ^ z));
+  const float4 ny = __ldg(nd + (r.ky ^ z)), fy = __ldg(nd + ((5 - r.ky) ^ z));
+  const float4 nz = __ldg(nd + (r.kz ^ z)), fz = __ldg(nd + ((7 - r.kz) ^ z));
+  const int4 child = __ldg(reinterpret_cast<const int4*>(nd + (6 ^ z)));
+  const float ax[4] = {nx.x, nx.y, nx.z, nx.w}, ay[4] = {ny.x, ny.y, ny.z, ny.w}, az[4] = {nz.x, nz.y, nz.z, nz.w};
+  const float bx[4] = {fx.x, fx.y, fx.z, fx.w}, by[4] = {fy.x, fy.y, fy.z, fy.w}, bz[4] = {fz.x, fz.y, fz.z, fz.w};
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const float x0 = (lx[k] - o.x) * inv.x, x1 = (hx[k] - o.x) * inv.x;
-    const float y0 = (ly[k] - o.y) * inv.y, y1 = (hy[k] - o.y) * inv.y;
-    const float z0 = (lz[k] - o.z) * inv.z, z1 = (hz[k] - o.z) * inv.z;
-    const float tn = fmax3(fminf(x0, x1), fminf(y0, y1), fmaxf(fminf(z0, z1), 0.0f));
-    const float tf = fmin3(fmaxf(x0, x1), fmaxf(y0, y1), fminf(fmaxf(z0, z1), tmax));
-    t[k] = (ch[k] != BVH4_EMPTY && tn <= tf * 1.00000024f) ? tn : __int_as_float(0x7fffffff);
+    t[k] = fmax3(__fmaf_rn(ax[k], r.ix, r.nx), __fmaf_rn(ay[k], r.iy, r.ny), fmaxf(__fmaf_rn(az[k], r.iz, r.nz), 0.0f));
+    e[k] = 1.0000005f * fmin3(__fmaf_rn(bx[k], r.ix, r.fx), __fmaf_rn(by[k], r.iy, r.fy),
+                              fminf(__fmaf_rn(bz[k], r.iz, r.fz), tmax));
   }
+  return child;
 }
 
-// Any hit with 0 < t < tmax over the 4-wide BVH.
-__device__ __forceinline__ bool trace_any4(const DevScene& s, f3 o, f3 d, float tmax, TraceWork& w) {
-  float th;
-  if (s.n_prims == 1) return hit_prim(s.prims, 0, o, d, tmax, th, w);
-  const f3 inv = mk3(1.0f / d.x, 1.0f / d.y, 1.0f / d.z);
-  int stack[STACK];
-  int sp = 0;
-  int node = 0;
-  for (int visits = 0; visits < s.n_nodes4; ++visits) {
-    if (!trav_ok(node >= 0 && node < s.n_nodes4, MARS_CHECK_NODE, w)) break;
-    const Bvh4Node nd = s.nodes4[node];
-    w.nodes += 2;
-    float t[4];
-    box4_entry(nd, o, inv, tmax, t);
-    const int ch[4] = {nd.child.x, nd.child.y, nd.child.z, nd.child.w};
-    int next = -1;
-    unsigned leaves = 0;  // admitted leaf children, tested below in child order
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (!(t[k] <= tmax)) continue;
-      if (ch[k] < 0) {
-        leaves |= 1u << k;
-      } else if (next < 0) {
-        next = ch[k];
-      } else if (sp < STACK) {
-        stack[sp++] = ch[k];
+// Closest hit of one ray over the 4-wide hierarchy, one step at a time, so that
+// a warp can choose what its lanes do together (see trace_pool).  `cur` is
+// what the ray looks at next: an inner node (>= 0), a primitive ~cur (< 0), or
+// TRAV_DONE.
+constexpr int TRAV_DONE = (int)0x80000000;
+
+// nearest-first order of up to four children: a key holds a met child's entry
+// distance (the bits of a non-negative float order like it) with the child's
+// slot in the two lowest bits, or all ones
+__device__ __forceinline__ void sort4(unsigned k[4]) {
+  auto cas = [](unsigned& a, unsigned& b) {
+    const unsigned lo = min(a, b), hi = max(a, b);
+    a = lo;
+    b = hi;
+  };
+  cas(k[0], k[1]);
+  cas(k[2], k[3]);
+  cas(k[0], k[2]);
+  cas(k[1], k[3]);
+  cas(k[1], k[2]);
+}
+__device__ __forceinline__ int pick4(int4 c, unsigned k) {
+  const int a = (k & 1u) ? c.y : c.x, b = (k & 1u) ? c.w : c.z;
+  return (k & 2u) ? b : a;
+}
+
+struct ClosestRay {
+  f3 o, d;
+  SlabRay r;
+  float t_best;
+  int best, cur, sp;
+
+  __device__ __forceinline__ void start(f3 o_, f3 d_) {
+    o = o_;
+    d = d_;
+    r = slab_ray(o, d);
+    t_best = __int_as_float(0x7f800000);
+    best = -1;
+    cur = 0;
+    sp = 0;
+  }
+  // the nearest entry left on the stack that can still hold a nearer hit
+  __device__ __forceinline__ void pop(const uint2* stack) {
+    cur = TRAV_DONE;
+    while (sp > 0) {
+      const uint2 q = stack[--sp];
+      if (__uint_as_float(q.x & ~3u) <= t_best) {
+        cur = (int)q.y;
+        break;
       }
     }
-    // one copy of the primitive test for all of them (lanes share it)
-    while (leaves) {
-      const int k = __ffs(leaves) - 1;
-      leaves &= leaves - 1;
-      const int c = k == 0 ? ch[0] : (k == 1 ? ch[1] : (k == 2 ? ch[2] : ch[3]));
-      if (!trav_ok(~c < s.n_prims, MARS_CHECK_PRIM, w)) return false;
-      if (hit_prim(s.prims, ~c, o, d, tmax, th, w)) return true;
-    }
-    if (next >= 0) {
-      node = next;
-    } else {
-      if (sp == 0) break;
-      node = stack[--sp];
-    }
   }
-  return false;
+  // visit inner node cur: the nearest met child is looked at next, the others
+  // (inner nodes and primitives alike) are pushed farthest first
+  __device__ __forceinline__ void node_step(const DevScene& s, uint2* stack, TraceWork& w) {
+    if (!trav_ok(cur < s.n_nodes4, MARS_CHECK_NODE, w)) { cur = TRAV_DONE; return; }
+    w.nodes += 2;
+    float t[4], e[4];
+    const int4 ch = box4(reinterpret_cast<const float4*>(s.nodes4), cur, r, t_best, t, e);
+    unsigned key[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      key[k] = t[k] <= e[k] ? ((__float_as_uint(t[k]) & ~3u) | (unsigned)k) : 0xffffffffu;
+    sort4(key);
+#pragma unroll
+    for (int k = 3; k >= 1; --k)
+      if (key[k] != 0xffffffffu) stack[sp++] = make_uint2(key[k], (unsigned)pick4(ch, key[k]));
+    if (key[0] != 0xffffffffu)
+      cur = pick4(ch, key[0]);
+    else
+      pop(stack);
+  }
+  // test primitive ~cur; ties in t go to the lower index, as in a scan in index order
+  __device__ __forceinline__ void leaf_step(const DevScene& s, uint2* stack, TraceWork& w) {
+    const int p = ~cur;
+    if (!trav_ok(p < s.n_prims, MARS_CHECK_PRIM, w)) { cur = TRAV_DONE; return; }
+    float t;
+    if (hit_prim(s.prims, p, o, d, t_best * 1.0000002f + 1e-30f, t, w) && (t < t_best || (t == t_best && p < best))) {
+      t_best = t;
+      best = p;
+    }
+    pop(stack);
+  }
+};
+
+// Any hit with 0 < t < tmax.  The children met are looked at in slot order (the
+// hierarchy's own order measured faster than nearest or farthest first).
+struct AnyRay {
+  f3 o, d;
+  SlabRay r;
+  float tmax;
+  int cur, sp;
+  bool hit;
+
+  __device__ __forceinline__ void start(f3 o_, f3 d_, float tmax_) {
+    o = o_;
+    d = d_;
+    tmax = tmax_;
+    r = slab_ray(o, d);
+    cur = 0;
+    sp = 0;
+    hit = false;
+  }
+  __device__ __forceinline__ void node_step(const DevScene& s, int* stack, TraceWork& w) {
+    if (!trav_ok(cur < s.n_nodes4, MARS_CHECK_NODE, w)) { cur = TRAV_DONE; return; }
+    w.nodes += 2;
+    float t[4], e[4];
+    const int4 c4 = box4(reinterpret_cast<const float4*>(s.nodes4), cur, r, tmax, t, e);
+    const int ch[4] = {c4.x, c4.y, c4.z, c4.w};
+    int next = TRAV_DONE;
+#pragma unroll
+    for (int k = 3; k >= 0; --k) {
+      if (!(t[k] <= e[k])) continue;
+      if (next != TRAV_DONE) stack[sp++] = next;
+      next = ch[k];
+    }
+    if (next == TRAV_DONE && sp > 0) next = stack[--sp];
+    cur = next;
+  }
+  __device__ __forceinline__ void leaf_step(const DevScene& s, int* stack, TraceWork& w) {
+    const int p = ~cur;
+    cur = TRAV_DONE;
+    if (!trav_ok(p < s.n_prims, MARS_CHECK_PRIM, w)) return;
+    float t;
+    if (hit_prim(s.prims, p, o, d, tmax, t, w))
+      hit = true;
+    else if (sp > 0)
+      cur = stack[--sp];
+  }
+};
+
+// Closest hit of one ray by one thread (light subpaths): the steps of
+// ClosestRay in the order the ray needs them.
+__device__ __forceinline__ int trace_closest(const DevScene& s, f3 o, f3 d, float& t_best, TraceWork& w) {
+  uint2 stack[STACK];
+  ClosestRay q;
+  q.start(o, d);
+  while (q.cur != TRAV_DONE) {
+    if (q.cur >= 0)
+      q.node_step(s, stack, w);
+    else
+      q.leaf_step(s, stack, w);
+  }
+  t_best = q.t_best;
+  return q.best;
 }
 
-// Any hit with 0 < t < tmax.
+// Any hit of one ray by one thread (connections of light subpaths).
 __device__ __forceinline__ bool trace_any(const DevScene& s, f3 o, f3 d, float tmax, TraceWork& w) {
-  float t;
-  if (s.n_prims == 1) return hit_prim(s.prims, 0, o, d, tmax, t, w);
-  const f3 inv = mk3(1.0f / d.x, 1.0f / d.y, 1.0f / d.z);
   int stack[STACK];
-  int sp = 0;
-  int node = 0;
-  for (int visits = 0; visits < s.n_prims; ++visits) {
-    if (!trav_ok(node >= 0 && node < s.n_prims - 1, MARS_CHECK_NODE, w)) break;
-    const BvhNode nd = s.nodes[node];
-    ++w.nodes;
-    const float tl = box_entry(nd.a, nd.b, o, inv, tmax);
-    const float tr = box_entry(nd.c, nd.d, o, inv, tmax);
-    const int cl = __float_as_int(nd.a.w), cr = __float_as_int(nd.b.w);
-    bool vl = tl <= tmax, vr = tr <= tmax;
-    if (vl && cl < 0) {
-      if (hit_prim(s.prims, ~cl, o, d, tmax, t, w)) return true;
-      vl = false;
-    }
-    if (vr && cr < 0) {
-      if (hit_prim(s.prims, ~cr, o, d, tmax, t, w)) return true;
-      vr = false;
-    }
-    if (vl && vr) {
-      if (sp < STACK) stack[sp++] = cr;
-      node = cl;
-    } else if (vl) {
-      node = cl;
-    } else if (vr) {
-      node = cr;
-    } else {
-      if (sp == 0) break;
-      node = stack[--sp];
-    }
+  AnyRay q;
+  q.start(o, d, tmax);
+  while (q.cur != TRAV_DONE) {
+    if (q.cur >= 0)
+      q.node_step(s, stack, w);
+    else
+      q.leaf_step(s, stack, w);
   }
-  return false;
+  return q.hit;
 }
 
 // geometric unit normal at p on primitive i

@@ -41,15 +41,20 @@ struct BvhNode {
   float4 a, b, c, d;
 };
 
-// 4-wide BVH node (collapsed from the binary LBVH on the host): the boxes of up
-// to four children as structure of arrays, one float4 per coordinate, and the
-// children: >= 0 internal node, < 0 primitive ~child, BVH4_EMPTY unused.
-constexpr int BVH4_EMPTY = 0x7fffffff;
+// 4-wide BVH node, what every traversal visits (collapsed from the binary BVH
+// on the host): the boxes of up to four children as structure of arrays, one
+// float4 per coordinate, and the children: >= 0 internal node, < 0 primitive
+// ~child; an unused slot holds an inverted infinite box.  On the device the
+// eight float4 of node n are permuted: float4 j at place j ^ (n & 7).
 struct Bvh4Node {
   float4 lox, loy, loz, hix, hiy, hiz;
   int4 child;
   float4 pad;
 };
+
+// entries of a traversal's stack: no path of the 4-wide hierarchy leaves more
+// pending (checked when it is collapsed)
+constexpr int TRAVERSAL_STACK = 64;
 
 // Material: m0 = (type, alpha, reflective, emissive), m1 = (colour rgb, 0),
 // m2 = (emitted radiance rgb, 0).
@@ -57,7 +62,6 @@ struct Bvh4Node {
 //        l3 = (unit normal xyz, primitive index bits), l4 = (radiance rgb, 0).
 struct DevScene {
   const float4* prims;
-  const BvhNode* nodes;
   const Bvh4Node* nodes4;
   int n_nodes4;
   const float4* mats;
@@ -85,11 +89,10 @@ struct DevScene {
 //   V4 = (Le luminance, 1/S_beta, parent cell, bin)
 //   S  = (sample value xyz, cost)
 // NEE shadow rays of wave d occupy [sbase[d], sbase[d] + scount[d]) of a second
-// arena: SH0 = (origin xyz, tmax; < 0: nothing to trace), SH1 = (direction, -),
-// SH2 = (sample value if visible, -), zeroed by the shadow kernel when occluded.
-// Only samples with a nonzero value need a ray: their slots are listed in
-// SL[sbase[d], sbase[d] + slcount[d]) (a compacted work list), and SH0/SH1 are
-// written for them alone.
+// arena: SH2 = (sample value if visible, -), zeroed by the shadow kernel when
+// occluded.  Only samples with a nonzero value need a ray: those rays are
+// listed, SH0 = (origin xyz, tmax), SH1 = (direction, slot of the sample's
+// value) at [sbase[d], sbase[d] + slcount[d]).
 //
 // With light connections (MARS_TECH_LIGHT) a ray carries the running sums of
 // the whole-path weights instead of the guided technique's fields:
@@ -113,7 +116,7 @@ struct DevScene {
 // written by the connection kernel.
 constexpr int NR = 5, NV = 5, NSH = 3, NLJ = 8, NLV = 6;
 constexpr int SLOT_BYTES = (NR + NV + 1) * 16 + 8 + 4;  // per ray slot
-constexpr int SHADOW_BYTES = NSH * 16 + 4;          // per shadow-ray slot
+constexpr int SHADOW_BYTES = NSH * 16;              // per shadow-ray slot
 // R5 per ray slot, LJ and LR per connection slot, LV and LC per light vertex
 // slot (as many of each as ray slots)
 constexpr int LIGHT_SLOT_BYTES = 16 + (NLJ + 1) * 16 + (NLV + 1) * 16;
@@ -124,7 +127,6 @@ struct Arena {
   float4* S;
   float* M;   // path multiplicity of the ray (product of the budgets that drew its path)
   float4* SH[NSH];
-  unsigned int* SL;
   float4* R5;        // light connections only
   float4* LJ[NLJ];
   float4* LR;
@@ -155,6 +157,8 @@ struct DevCounters {
   unsigned long long lbase[MAXD + 2];    // light connection samples of wave d
   unsigned long long lcount[MAXD + 2];
   unsigned long long vcount[MAXD + 2];   // light subpath vertices of wave d's samples
+  unsigned long long trace_next[MAXD + 2];   // rays of wave d taken from the wave's shared pool
+  unsigned long long shadow_next[MAXD + 2];  // shadow rays of wave d taken from theirs
   unsigned long long light_rays, conn_rays;  // light-subpath closest hits, connection rays (every launch)
   unsigned long long light_entries;          // light connection samples of committed tiles
   unsigned long long light_vertex_entries;   // light subpath vertices of committed tiles
@@ -304,6 +308,10 @@ cudaError_t launch_update(const DevCache& c, int num_sms, cudaStream_t st);
 cudaError_t launch_leaf_samples(const DevCache& c, cudaStream_t st);
 cudaError_t launch_octree_refine(const DevCache& c, int num_sms, cudaStream_t st);
 // scene build (scene.cu)
+// the 4-wide form of a binary hierarchy over n primitives (boxes: 2 float4 per
+// primitive), in device order; entries: the traversal stack's largest need
+bool collapse_bvh4(const std::vector<BvhNode>& bin, const std::vector<float4>& boxes, int n, std::vector<Bvh4Node>& out,
+                   int* entries);
 // SAH build on the host from the primitive boxes (2 float4 per primitive):
 // n - 1 internal nodes, root 0; false if n < 2 (scene.cu)
 bool build_bvh_sah(const std::vector<float4>& boxes, int n, std::vector<BvhNode>& nodes);

@@ -136,6 +136,8 @@ __global__ void k_tile_init(DevCounters* ctr, const IterArgs* __restrict__ itp) 
     ctr->lbase[t] = 0;
     ctr->lcount[t] = 0;
     ctr->vcount[t] = 0;
+    ctr->trace_next[t] = 0;
+    ctr->shadow_next[t] = 0;
   }
   if (t == 0) {
     ctr->overflow = 0;
@@ -209,43 +211,159 @@ __global__ void k_merge_lanes(DevCounters* dst, DevCounters* src) {
 }
 
 // ------------------------------------------------------------------ trace
+// The rays of a wave as its warps take them: chunks of 32, the first the warp's
+// own, the others from a counter that the grid's warps share.  The two records
+// of a chunk's rays are copied to shared memory one chunk ahead (cp.async), so
+// that a lane that takes a ray does not wait for device memory.
+struct RayStage {
+  float4 r[2][2][32];  // [buffer][record][ray of the chunk]
+};
+struct RayPool {
+  const float4 *g0, *g1;  // the wave's records (null: rays without records)
+  unsigned long long* counter;
+  RayStage* st;
+  unsigned n, base, cnt, off, nbase, ncnt;  // wave, current chunk (rays used: off), next chunk
+  int buf;
+
+  __device__ __forceinline__ void load(unsigned b, unsigned c, int which, int lane) {
+    if (g0 && (unsigned)lane < c) {
+      const unsigned d0 = (unsigned)__cvta_generic_to_shared(&st->r[which][0][lane]);
+      const unsigned d1 = (unsigned)__cvta_generic_to_shared(&st->r[which][1][lane]);
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d0), "l"(g0 + b + lane) : "memory");
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d1), "l"(g1 + b + lane) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  __device__ __forceinline__ void grab(int lane) {
+    const unsigned long long own = ((gridDim.x * (unsigned long long)blockDim.x) >> 5) * 32ull;
+    nbase = ncnt = 0;
+    if ((unsigned long long)n > own) {
+      unsigned long long b = 0;
+      if (lane == 0) b = atomicAdd(counter, 32ull);
+      b = own + __shfl_sync(FULL, b, 0);
+      if (b < n) {
+        nbase = (unsigned)b;
+        ncnt = min(32u, n - nbase);
+      }
+    }
+  }
+  __device__ __forceinline__ RayPool(const float4* g0_, const float4* g1_, unsigned n_, unsigned long long* counter_,
+                                     RayStage* st_, int lane)
+      : g0(g0_), g1(g1_), counter(counter_), st(st_), n(n_), off(0), buf(0) {
+    const unsigned long long b = ((blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) >> 5) * 32ull;
+    base = b < n ? (unsigned)b : 0u;
+    cnt = b < n ? min(32u, n - base) : 0u;
+    load(base, cnt, 0, lane);
+    grab(lane);
+    load(nbase, ncnt, 1, lane);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
+  }
+  __device__ __forceinline__ bool dry() const { return off >= cnt && ncnt == 0; }
+  // a ray of the current chunk for every lane of `want`, as far as the chunk
+  // goes: its index in the chunk, or -1
+  __device__ __forceinline__ int take(unsigned want, int lane) {
+    if (off >= cnt && ncnt > 0) {
+      __syncwarp();
+      base = nbase;
+      cnt = ncnt;
+      off = 0;
+      grab(lane);
+      load(nbase, ncnt, buf, lane);
+      buf ^= 1;
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncwarp();
+    }
+    const unsigned k = off + (unsigned)__popc(want & ((1u << lane) - 1u));
+    off = min(cnt, off + (unsigned)__popc(want));
+    return ((want >> lane) & 1u) && k < cnt ? (int)k : -1;
+  }
+};
+
+// Traversal of the pool's rays, a warp's lanes each on a ray of their own.
+// Divergence and the latency of a step's chain of loads and comparisons bound
+// it, not arithmetic or bandwidth: rays of a wave need between a few and a
+// hundred steps, and inner nodes and primitives run other code.  So lanes whose
+// ray has ended take new rays as soon as REFILL of them wait (the others go on
+// meanwhile), and each turn runs one kind of step: primitives when more than a
+// third of the busy lanes are at one, else nodes (primitives shorten the rays
+// they hit; any turn's kind left to the nodes alone was 25 % slower).
+// Against one ray per thread from start to end over the binary hierarchy:
+// guided room 512^2, first bounce, 0.67M rays: 12.0 -> 16.9 active lanes per
+// instruction, 76.6M -> 66.6M warp instructions, 117 -> 108 us; iterations of
+// the 524k-triangle scene at 2048^2 11.7 -> 10.8 ms, of the bidirectional
+// 131k-triangle scene at 1024^2 4.9 -> 4.3 ms.  REFILL 4 to 16 measure alike,
+// 24 and 32 slower on large scenes (11.6 and 11.1 ms).
+// start(k, o4, d4, ray) prepares ray k of the wave and returns whether it is
+// traced; done(k, ray) stores its result.
+constexpr int REFILL = 8;
+template <class Ray, class Entry, class Start, class Done>
+__device__ __forceinline__ void trace_pool(const DevScene& s, RayPool& pool, Entry* stack, TraceWork& tw, int lane,
+                                           Start start, Done done) {
+  Ray q;
+  q.cur = TRAV_DONE;
+  unsigned li = 0;
+  while (true) {
+    const unsigned idle = __ballot_sync(FULL, q.cur == TRAV_DONE);
+    if (idle == FULL || (__popc(idle) >= REFILL && !pool.dry())) {
+      const int k = pool.take(idle, lane);
+      if (k >= 0) {
+        li = pool.base + (unsigned)k;
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (!start(li, pool.g0 ? pool.st->r[pool.buf][0][k] : z, pool.g0 ? pool.st->r[pool.buf][1][k] : z, q))
+          q.cur = TRAV_DONE;
+      }
+      if (pool.dry() && __ballot_sync(FULL, q.cur != TRAV_DONE) == 0u) break;
+    }
+    const unsigned nodes = __ballot_sync(FULL, q.cur >= 0);
+    const unsigned leaves = __ballot_sync(FULL, q.cur < 0 && q.cur != TRAV_DONE);
+    if (__popc(nodes) >= 2 * __popc(leaves)) {
+      if (q.cur >= 0) {
+        q.node_step(s, stack, tw);
+        if (q.cur == TRAV_DONE) done(li, q);
+      }
+    } else if (q.cur < 0 && q.cur != TRAV_DONE) {
+      q.leaf_step(s, stack, tw);
+      if (q.cur == TRAV_DONE) done(li, q);
+    }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 template <int MINB>
 __global__ void __launch_bounds__(MAX_WAVE_THREADS, MINB) k_trace(const DevScene s, const DevCache c, const Arena a,
                                                          const IterArgs* __restrict__ itp, const int d) {
   const IterArgs it = *itp;
-  const DevCounters* ctr = c.ctr;
+  DevCounters* ctr = c.ctr;
   // after an overflow some slots of this wave were never written: stop, the
   // tile is re-rendered in smaller pieces
   if (ctr->overflow) return;
   const Wave w = wave_of(ctr, a, d);
   const Rng rng{it.seed, it.job, it.iteration};
   TraceWork tw;
-  // One ray per thread, grid-stride.  (A persistent variant that refills the
-  // lanes of finished rays from a warp-private pool measured 1.7x slower: the
-  // refill bookkeeping costs more than the idle lanes it recovers.)
-  for (unsigned long long li = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; li < w.n;
-       li += gridDim.x * (unsigned long long)blockDim.x) {
-    const unsigned long long i = w.base + li;
-    if (!chk(i < a.cap, MARS_CHECK_ARENA, c.ctr)) break;
-    f3 o, dir;
-    bool alive = true;
-    if (d == 1) {
-      camera_ray(s, rng, (uint32_t)(it.tile_begin + li), o, dir);
-    } else {
-      const float4 r0 = a.R[0][i], r1 = a.R[1][i];
-      o = xyz(r0);
-      dir = xyz(r1);
-      alive = r1.w > 0.0f;  // A = beta_t p_t is 0 for a drawn sample that is not traced
-    }
-    float t = 0.0f;
-    int prim = -2;  // -2: not traced, -1: traced and missed
-    // binary traversal: measured faster for closest hits than the 4-wide one,
-    // whose per-node ordering and eager leaf tests cost more than the halved
-    // node visits save; shadow rays use the 4-wide BVH
-    if (alive) prim = trace_closest(s, o, dir, t, tw);
-    a.H[i] = make_float2(t, __int_as_float(prim));
-  }
-  flush_work(tw, c.ctr->trace_work[0], c.ctr);
+  extern __shared__ RayStage ray_stage[];
+  const int lane = threadIdx.x & 31;
+  uint2 stack[STACK];
+  const bool camera = d == 1;
+  RayPool pool(camera ? nullptr : a.R[0] + w.base, camera ? nullptr : a.R[1] + w.base, (unsigned)w.n,
+               &ctr->trace_next[d], ray_stage + (threadIdx.x >> 5), lane);
+  // the hit record's primitive: -1 traced and missed, -2 not traced
+  trace_pool<ClosestRay>(
+      s, pool, stack, tw, lane,
+      [&](unsigned li, float4 r0, float4 r1, ClosestRay& q) {
+        if (!chk(w.base + li < a.cap, MARS_CHECK_ARENA, ctr)) return false;
+        f3 o = xyz(r0), dir = xyz(r1);
+        if (camera) {
+          camera_ray(s, rng, (uint32_t)it.tile_begin + li, o, dir);
+        } else if (!(r1.w > 0.0f)) {  // A = beta_t p_t is 0 for a drawn sample that is not traced
+          a.H[w.base + li] = make_float2(0.0f, __int_as_float(-2));
+          return false;
+        }
+        q.start(o, dir);
+        return true;
+      },
+      [&](unsigned li, const ClosestRay& q) { a.H[w.base + li] = make_float2(q.t_best, __int_as_float(q.best)); });
+  flush_work(tw, ctr->trace_work[0], ctr);
 }
 
 // ------------------------------------------------------------------ shade
@@ -656,9 +774,8 @@ __global__ void __launch_bounds__(MAX_WAVE_THREADS, MINB) k_shade(const DevScene
         if (trace) {
           const unsigned long long pos = sbase + lb + (unsigned long long)__popc(need & ((1u << lane) - 1u));
           if (pos < a.scap) {
-            a.SL[pos] = (unsigned int)j;
-            a.SH[0][j] = f4(xo, tmax);
-            a.SH[1][j] = f4(wi, 0.0f);
+            a.SH[0][pos] = f4(xo, tmax);
+            a.SH[1][pos] = f4(wi, __uint_as_float((unsigned int)j));
           }
         }
       }
@@ -802,26 +919,33 @@ __global__ void __launch_bounds__(MAX_WAVE_THREADS, MINB) k_shade(const DevScene
 }
 
 // ----------------------------------------------------------------- shadow
+// the listed shadow rays of wave d: SH0, SH1[sbase, sbase + slcount) (at most
+// scount of them), each with the slot of its sample's value
 template <int MINB>
 __global__ void __launch_bounds__(MAX_WAVE_THREADS, MINB) k_shadow(const DevScene s, const DevCache c, const Arena a,
                                                            const int d) {
-  const DevCounters* ctr = c.ctr;
+  DevCounters* ctr = c.ctr;
   if (ctr->overflow) return;
-  // the listed shadow rays of wave d: SL[sbase, sbase + slcount), slot indices
-  // into the wave's shadow region (at most scount of them)
   const unsigned long long sb = ctr->sbase[d], sl = ctr->slcount[d];
   const unsigned long long n = sl < a.scap - sb ? sl : a.scap - sb;
   TraceWork tw;
-  for (unsigned long long k = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; k < n;
-       k += gridDim.x * (unsigned long long)blockDim.x) {
-    const unsigned long long j = a.SL[sb + k];
-    if (!chk(j < a.scap, MARS_CHECK_SHADOW, c.ctr)) continue;
-    const float4 s0 = a.SH[0][j];
-    if (!(s0.w > 0.0f)) continue;
-    const float4 s1 = a.SH[1][j];
-    if (trace_any4(s, xyz(s0), xyz(s1), s0.w, tw)) a.SH[2][j] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  flush_work(tw, c.ctr->trace_work[1], c.ctr);
+  extern __shared__ RayStage ray_stage[];
+  const int lane = threadIdx.x & 31;
+  int stack[STACK];
+  unsigned j = 0;
+  RayPool pool(a.SH[0] + sb, a.SH[1] + sb, (unsigned)n, &ctr->shadow_next[d], ray_stage + (threadIdx.x >> 5), lane);
+  trace_pool<AnyRay>(
+      s, pool, stack, tw, lane,
+      [&](unsigned, float4 s0, float4 s1, AnyRay& q) {
+        j = __float_as_uint(s1.w);
+        if (!(s0.w > 0.0f)) return false;
+        q.start(xyz(s0), xyz(s1), s0.w);
+        return true;
+      },
+      [&](unsigned, const AnyRay& q) {
+        if (q.hit && chk(j < a.scap, MARS_CHECK_SHADOW, ctr)) a.SH[2][j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      });
+  flush_work(tw, ctr->trace_work[1], ctr);
 }
 
 // ---------------------------------------------------------------- reverse
@@ -1075,6 +1199,7 @@ __global__ void __launch_bounds__(MAX_WAVE_THREADS, MINB) k_reverse(const DevSce
   }
 }
 
+size_t trace_smem(int threads) { return (size_t)(threads / 32) * sizeof(RayStage); }
 size_t shade_smem(int threads) { return (size_t)(threads / 32) * sizeof(ShadeWarpCtx); }
 
 // Register-cap variants of every wave kernel, compiled with
@@ -1114,14 +1239,14 @@ cudaError_t wave_occupancy(const int threads[WAVE_KERNELS], const int variant[WA
                            int blocks_per_sm[WAVE_KERNELS]) {
   cudaError_t e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[WK_TRACE], trace_fn(variant[WK_TRACE]),
-                                                         threads[WK_TRACE], 0)) != cudaSuccess)
+                                                         threads[WK_TRACE], trace_smem(threads[WK_TRACE]))) != cudaSuccess)
     return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[WK_SHADE], shade_fn(variant[WK_SHADE]),
                                                          threads[WK_SHADE], shade_smem(threads[WK_SHADE]))) !=
       cudaSuccess)
     return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[WK_SHADOW], shadow_fn(variant[WK_SHADOW]),
-                                                         threads[WK_SHADOW], 0)) != cudaSuccess)
+                                                         threads[WK_SHADOW], trace_smem(threads[WK_SHADOW]))) != cudaSuccess)
     return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm[WK_REVERSE], reverse_fn(variant[WK_REVERSE]),
                                                        threads[WK_REVERSE], 0);
@@ -1162,7 +1287,7 @@ cudaError_t launch_tile(const DevScene& s, const DevCache& c, const Arena& a, co
   cudaStream_t lside = side2 ? side2 : side;
   bool any_shadow = false, any_light = false;
   for (int d = 1; d <= D; ++d) {
-    trace_fn(L.variant[WK_TRACE])<<<G(WK_TRACE, d), tT, 0, st>>>(s, c, a, it, d);
+    trace_fn(L.variant[WK_TRACE])<<<G(WK_TRACE, d), tT, trace_smem(tT), st>>>(s, c, a, it, d);
     if (ev) cudaEventRecord(ev[2 * (d - 1) + 1], st);
     shade_fn(L.variant[WK_SHADE], bd)<<<G(WK_SHADE, d), tS, smS, st>>>(s, c, a, it, d);
     if (ev) cudaEventRecord(ev[2 * (d - 1) + 2], st);
@@ -1172,7 +1297,7 @@ cudaError_t launch_tile(const DevScene& s, const DevCache& c, const Arena& a, co
       cudaStreamWaitEvent(side, sync[d - 1], 0);
       any_shadow = true;
       if (ev) cudaEventRecord(ev[2 * D + 2 * (d - 1) + 1], side);
-      shadow_fn(L.variant[WK_SHADOW])<<<G(WK_SHADOW, d), tH, 0, side>>>(s, c, a, d);
+      shadow_fn(L.variant[WK_SHADOW])<<<G(WK_SHADOW, d), tH, trace_smem(tH), side>>>(s, c, a, d);
       if (ev) cudaEventRecord(ev[2 * D + 2 * (d - 1) + 2], side);
     }
     if (light) {

@@ -367,4 +367,101 @@ bool build_bvh_sah(const std::vector<float4>& boxes, int n, std::vector<BvhNode>
   return next == n - 1;
 }
 
+// ------------------------------------------------------- 4-wide hierarchy
+// A node's children are grown by replacing the internal child with the largest
+// box surface by its two children until there are four or only leaves remain.
+// A traversal looks at one met child next and pushes the others, so a path
+// leaves at most the sum of (children - 1) over its nodes pending; where that
+// exceeds the traversal's stack (no hierarchy of the builders has been seen to)
+// nodes keep the binary hierarchy's two children, one entry a level, and its
+// depth, at most 63 for the linear and kMaxDepth for the SAH build, bounds it.
+bool collapse_bvh4(const std::vector<BvhNode>& bin, const std::vector<float4>& boxes, int n, std::vector<Bvh4Node>& out,
+                   int* entries) {
+  struct Ch {
+    int id;              // >= 0 binary internal node, < 0 ~primitive
+    float lo[3], hi[3];
+  };
+  struct Todo {
+    int bk, slot, pending;  // binary node, 4-wide node, stack entries left when it is visited
+  };
+  auto kids = [&](int k, Ch* c) {
+    const BvhNode& b = bin[k];
+    int l, r;
+    std::memcpy(&l, &b.a.w, sizeof(int));
+    std::memcpy(&r, &b.b.w, sizeof(int));
+    c[0] = {l, {b.a.x, b.a.y, b.a.z}, {b.b.x, b.b.y, b.b.z}};
+    c[1] = {r, {b.c.x, b.c.y, b.c.z}, {b.d.x, b.d.y, b.d.z}};
+  };
+  auto area = [](const Ch& c) {
+    const double dx = c.hi[0] - c.lo[0], dy = c.hi[1] - c.lo[1], dz = c.hi[2] - c.lo[2];
+    return dx * dy + dy * dz + dz * dx;
+  };
+  for (int width : {4, 2}) {
+    int need = 0;
+    out.clear();
+    out.reserve(n);
+    std::vector<Todo> todo;
+    out.emplace_back();
+    todo.push_back({0, 0, 0});
+    while (!todo.empty()) {
+      const Todo t = todo.back();
+      todo.pop_back();
+      Ch set[4];
+      int m = 2;
+      if (n == 1) {
+        m = 1;
+        set[0] = {~0, {boxes[0].x, boxes[0].y, boxes[0].z}, {boxes[1].x, boxes[1].y, boxes[1].z}};
+      } else {
+        kids(t.bk, set);
+      }
+      while (m >= 2 && m < width) {
+        int best = -1;
+        double ba = -1.0;
+        for (int k = 0; k < m; ++k)
+          if (set[k].id >= 0 && area(set[k]) > ba) { ba = area(set[k]); best = k; }
+        if (best < 0) break;
+        Ch two[2];
+        kids(set[best].id, two);
+        set[best] = two[0];
+        set[m++] = two[1];
+      }
+      const int below = t.pending + m - 1;
+      need = std::max(need, below);
+      float lo[3][4], hi[3][4];
+      int ch[4];
+      for (int k = 0; k < 4; ++k) {
+        for (int a = 0; a < 3; ++a) {
+          lo[a][k] = k < m ? set[k].lo[a] : INFINITY;   // unused slot: an inverted box, met by no ray
+          hi[a][k] = k < m ? set[k].hi[a] : -INFINITY;
+        }
+        ch[k] = k < m ? set[k].id : ~0;
+        if (k < m && set[k].id >= 0) {
+          ch[k] = (int)out.size();
+          out.emplace_back();
+          todo.push_back({set[k].id, ch[k], below});
+        }
+      }
+      Bvh4Node& nd = out[t.slot];
+      nd.lox = make_float4(lo[0][0], lo[0][1], lo[0][2], lo[0][3]);
+      nd.loy = make_float4(lo[1][0], lo[1][1], lo[1][2], lo[1][3]);
+      nd.loz = make_float4(lo[2][0], lo[2][1], lo[2][2], lo[2][3]);
+      nd.hix = make_float4(hi[0][0], hi[0][1], hi[0][2], hi[0][3]);
+      nd.hiy = make_float4(hi[1][0], hi[1][1], hi[1][2], hi[1][3]);
+      nd.hiz = make_float4(hi[2][0], hi[2][1], hi[2][2], hi[2][3]);
+      nd.child = make_int4(ch[0], ch[1], ch[2], ch[3]);
+      nd.pad = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    *entries = need;
+    if (need <= TRAVERSAL_STACK) break;
+  }
+  // device order (see Bvh4Node)
+  for (size_t k = 0; k < out.size(); ++k) {
+    float4 raw[8], sw[8];
+    std::memcpy(raw, &out[k], sizeof(raw));
+    for (int j = 0; j < 8; ++j) sw[j ^ (int)(k & 7)] = raw[j];
+    std::memcpy(&out[k], sw, sizeof(sw));
+  }
+  return *entries <= TRAVERSAL_STACK;
+}
+
 }  // namespace mars
