@@ -17,12 +17,12 @@ LIB = os.path.join(PKG, "libmars.so")
 # the checked variant: the same sources with the kernels' index checks compiled in
 BUILD_CHECKED = os.path.join(PKG, "_build_checked")
 LIB_CHECKED = os.path.join(PKG, "libmars_checked.so")
-SOURCES = ["abi.cu", "render.cu", "bdpt.cu", "stats.cu", "scene.cu", "server.cu", "static_scratch.cu"]
+SOURCES = ["abi.cu", "render.cu", "tail.cu", "bdpt.cu", "stats.cu", "scene.cu", "server.cu", "static_scratch.cu"]
 # the wave kernels (traversal, shading, light subpaths, reverse pass) take
 # float32 division and square root to within 2 ulp instead of correctly
 # rounded (the cell of a point keeps the IEEE operations); the hierarchy
 # build, image statistics and count update keep IEEE float32 arithmetic
-APPROX_DIV_SQRT = {"render.cu", "bdpt.cu"}
+APPROX_DIV_SQRT = {"render.cu", "tail.cu", "bdpt.cu"}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -61,11 +61,12 @@ struct NvtxRange {
 struct GraphKey {
   bool update_estimate = false, drop = false, combine = false;
   int tiles = 0;
+  int tail = 0;
   float* dev_out = nullptr;
   int64_t r0 = 0, r1 = 0;  // pixel range (the image copy of a range is recorded with its bounds)
   WaveLaunch L{};
   bool operator==(const GraphKey& o) const {
-    return update_estimate == o.update_estimate && drop == o.drop && combine == o.combine && tiles == o.tiles &&
+    return update_estimate == o.update_estimate && drop == o.drop && combine == o.combine && tiles == o.tiles && tail == o.tail &&
            dev_out == o.dev_out && r0 == o.r0 && r1 == o.r1 && std::memcmp(&L, &o.L, sizeof(WaveLaunch)) == 0;
   }
 };
@@ -125,6 +126,11 @@ struct mars_cache {
   unsigned int* d_tile_status = nullptr;
   mars::DevCounters* h_ctr = nullptr;
   unsigned int* h_tile_status = nullptr;
+  uint4* d_tail_rounds = nullptr;  // one buffer per lane (see DevCache)
+  int tail_blocks = 0;             // resident blocks of k_tail (0: it is not used)
+  double tail_margin = 2.0;        // headroom of k_tail's slices over the last iteration's use
+  uint64_t last_wave[mars::MAXD + 2] = {};  // rays per depth of the last iteration
+  int64_t last_pixels = 0;                  // and its pixels
   int max_tiles = 0;
   int next_tiles = 1;
   int n_iterations = 0;

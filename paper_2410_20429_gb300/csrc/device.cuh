@@ -51,12 +51,44 @@ __device__ __forceinline__ f3 operator+(f3 a, f3 b) { return {a.x + b.x, a.y + b
 __device__ __forceinline__ f3 operator-(f3 a, f3 b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
 __device__ __forceinline__ f3 operator*(f3 a, float s) { return {a.x * s, a.y * s, a.z * s}; }
 __device__ __forceinline__ f3 mul(f3 a, f3 b) { return {a.x * b.x, a.y * b.y, a.z * b.z}; }
-__device__ __forceinline__ float dot(f3 a, f3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+// Sums of products.  The compiler may fuse either product of a * b + c * d into
+// the addition, and which one it takes depends on the code around it.
+// MARS_PIN_FMA spells out the choice it makes in the wave kernels, for a
+// translation unit whose kernels have to give their results bit for bit.
+#ifdef MARS_PIN_FMA
+__device__ __forceinline__ float sum2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ float diff2(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
+#else
+__device__ __forceinline__ float sum2(float a, float b, float c, float d) { return a * b + c * d; }
+__device__ __forceinline__ float diff2(float a, float b, float c, float d) { return a * b - c * d; }
+#endif
+__device__ __forceinline__ float sum3(float a, float b, float c, float d, float e, float f) {
+#ifdef MARS_PIN_FMA
+  return __fmaf_rn(e, f, sum2(a, b, c, d));
+#else
+  return a * b + c * d + e * f;
+#endif
+}
+__device__ __forceinline__ float dot(f3 a, f3 b) { return sum3(a.x, b.x, a.y, b.y, a.z, b.z); }
 __device__ __forceinline__ f3 cross(f3 a, f3 b) {
-  return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
+  return {diff2(a.y, b.z, a.z, b.y), diff2(a.z, b.x, a.x, b.z), diff2(a.x, b.y, a.y, b.x)};
+}
+__device__ __forceinline__ float length2_hit(f3 a) {
+#ifdef MARS_PIN_FMA
+  return __fmaf_rn(a.z, a.z, __fmaf_rn(a.y, a.y, __fmul_rn(a.x, a.x)));
+#else
+  return dot(a, a);
+#endif
+}
+// a u + b v (+ c w)
+__device__ __forceinline__ f3 span2(f3 a, float u, f3 b, float v) {
+  return {sum2(a.x, u, b.x, v), sum2(a.y, u, b.y, v), sum2(a.z, u, b.z, v)};
+}
+__device__ __forceinline__ f3 span3(f3 a, float u, f3 b, float v, f3 c, float w) {
+  return {sum3(a.x, u, b.x, v, c.x, w), sum3(a.y, u, b.y, v, c.y, w), sum3(a.z, u, b.z, v, c.z, w)};
 }
 __device__ __forceinline__ f3 normalize(f3 a) { return a * (1.0f / sqrtf(dot(a, a))); }
-__device__ __forceinline__ float lum(f3 c) { return 0.2126f * c.x + 0.7152f * c.y + 0.0722f * c.z; }
+__device__ __forceinline__ float lum(f3 c) { return sum3(0.2126f, c.x, 0.7152f, c.y, 0.0722f, c.z); }
 __device__ __forceinline__ bool nonzero(f3 c) { return c.x > 0.f || c.y > 0.f || c.z > 0.f; }
 
 // ------------------------------------------------------------ intersection
@@ -397,7 +429,7 @@ __device__ __forceinline__ int prim_material(const float4* __restrict__ prims, i
 struct Frame {
   f3 b1, b2, n;
   __device__ __forceinline__ f3 to_local(f3 w) const { return mk3(dot(w, b1), dot(w, b2), dot(w, n)); }
-  __device__ __forceinline__ f3 to_world(f3 l) const { return b1 * l.x + b2 * l.y + n * l.z; }
+  __device__ __forceinline__ f3 to_world(f3 l) const { return span3(b1, l.x, b2, l.y, n, l.z); }
 };
 __device__ __forceinline__ Frame make_frame(f3 n) {
   const float sign = copysignf(1.0f, n.z);
@@ -427,7 +459,7 @@ struct Mat {
 // Smith Lambda of a unit direction w (local frame): tan^2 = (x^2 + y^2) / z^2,
 // written without the cancellation of 1 - cos^2 in float32
 __device__ __forceinline__ float ggx_lambda(float a2, f3 w) {
-  const float t2 = (w.x * w.x + w.y * w.y) / (w.z * w.z);
+  const float t2 = sum2(w.x, w.x, w.y, w.y) / (w.z * w.z);
   return 0.5f * (-1.0f + sqrtf(1.0f + a2 * t2));
 }
 
@@ -447,7 +479,7 @@ __device__ __forceinline__ f3 bsdf_eval(const Mat& m, f3 wo, f3 wi, float& pdf) 
   if (woh <= 0.0f) return mk3(0.f, 0.f, 0.f);
   // 1 + cos^2(alpha^2 - 1) = sin^2 + alpha^2 cos^2 for a unit h: no cancellation
   // near the specular peak of a smooth surface
-  const float k = (h.x * h.x + h.y * h.y) + a2 * (h.z * h.z);
+  const float k = sum3(h.x, h.x, h.y, h.y, a2, h.z * h.z);
   const float D = a2 * INV_PI_F / (k * k);
   const float G = 1.0f / (1.0f + ggx_lambda(a2, wo) + ggx_lambda(a2, wi));
   const float sf = 1.0f - woh;

@@ -147,6 +147,9 @@ constexpr uint32_t F_EST = 1u << 25;
 // of the grid serialise
 constexpr int IMG_SLOTS = 32;
 
+// rounds a block of k_tail may take
+constexpr int TAIL_ROUNDS = 96;
+
 // Device-resident per-iteration counters.
 struct DevCounters {
   unsigned long long base[MAXD + 2];
@@ -220,6 +223,8 @@ struct DevCache {
   float4* img;          // [pixels] this iteration's image
   DevCounters* ctr;
   unsigned int* tile_status;  // [max tiles] overflow per tile of the current attempt
+  uint4* tail_rounds;         // k_tail's rounds: [blocks][TAIL_ROUNDS] (first child, rays, children, first root),
+                              // then [blocks] (rounds, -, -, -); one such buffer per lane
   // adaptive octree over the scene box (oct_nodes null: the uniform grid).
   // node >= 0: first of its 8 children (octant x | y << 1 | z << 2); < 0: leaf ~cell
   int* oct_nodes;       // [oct_cap_nodes]
@@ -276,10 +281,12 @@ int light_variants();
 
 // launch wrappers (render.cu)
 // it: device pointer to the tile's arguments
+// tail: the waves from this depth on run in k_tail, with tail_blocks blocks (0:
+// every wave in the wave kernels; always 0 with light connections)
 // side2: the light connection kernels' stream (light connections only; null:
 // they run on side); sync: D + 2 events
 cudaError_t launch_tile(const DevScene& s, const DevCache& c, const Arena& a, const IterArgs* it,
-                        const WaveLaunch& L, int64_t tile_pixels, cudaStream_t st, cudaStream_t side, cudaStream_t side2,
+                        const WaveLaunch& L, int64_t tile_pixels, int tail, int tail_blocks, cudaStream_t st, cudaStream_t side, cudaStream_t side2,
                         const cudaEvent_t* sync, cudaEvent_t* ev);
 // adds a second tile lane's iteration totals into the first lane's counters
 cudaError_t launch_merge_lanes(DevCounters* dst, DevCounters* src, cudaStream_t st);
@@ -290,7 +297,13 @@ int wave_variants(int kernel);                    // compiled register-cap varia
 int wave_variant_registers(int kernel, int v);    // its register cap (0: the library's choice)
 bool wave_variant_repeats(int kernel, int v);     // the same code as variant 0
 bool wave_threads_ok(int threads);
-int tile_launches(int max_depth, int techniques);  // kernels launch_tile issues
+int tile_launches(int max_depth, int techniques, int tail);  // kernels launch_tile issues
+// the waves from depth k on (tail.cu): forward, and in reverse over the same grid
+int tail_occupancy();  // resident blocks per SM
+void launch_tail(const DevScene& s, const DevCache& c, const Arena& a, const IterArgs* it, int k, int blocks,
+                 cudaStream_t st);
+void launch_tail_reverse(const DevScene& s, const DevCache& c, const Arena& a, const IterArgs* it, int k, int blocks,
+                         cudaStream_t st);
 // image statistics (stats.cu)
 // it: device pointer to the iteration's arguments (n_prev, outlier, drop_k,
 // combine); drop / combine: whether the brightest-pixel rejection and the

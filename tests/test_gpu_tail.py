@@ -1,0 +1,102 @@
+"""The deep waves in two kernels (csrc/render.cu, k_tail and k_tail_reverse)
+against the wave kernels: a profiled iteration renders with the wave kernels
+alone, so the same iteration of the same state with and without `profile` gives
+the same image and counters, and statistics that differ by the order of their
+float additions only."""
+import numpy as np
+import pytest
+
+import mars_workloads as W
+
+pytestmark = pytest.mark.gpu
+
+TECH3 = W.TECH_BSDF | W.TECH_NEE | W.TECH_GUIDED
+KEYS = ("rays", "vertices", "estimator_vertices", "wave_entries", "shadow_entries", "shadow_traced", "wave_rays",
+        "trace_work")
+
+
+@pytest.fixture(scope="module")
+def mars():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_2410_20429_gb300 import build as B
+    B.build()
+    import paper_2410_20429_gb300 as M
+    return M
+
+
+def _pair(mars, w, h, D, tech, lo, hi, cap=0, lanes=2):
+    """(profiled, not profiled) results of one MARS iteration from the same state."""
+    import torch
+    sc = W.guided_room_scene(2, w, h, n_spheres=24)
+    stream = torch.cuda.Stream()
+    scene = mars.Scene(sc, stream=stream)
+    c = mars.Cache(scene, 6, tech, D, arena_capacity=cap, lanes=lanes, stream=stream)
+    q_rr, q_s, valid = W.random_count_fields(c.n_cells, seed=31, lo=lo, hi=hi)
+    est = W.random_pixel_estimate(sc.n_pixels, seed=32, lo=0.2, hi=0.5)
+    img = torch.zeros(3 * sc.n_pixels, dtype=torch.float32, device="cuda")
+    out = []
+    for profile in (True, False):
+        st = dict(q_rr=q_rr, q_s=q_s, valid=valid, pixel_estimate=est, has_estimate=True, n_iterations=1,
+                  stats=np.zeros((c.n_cells, 3, 8)))
+        if tech & W.TECH_GUIDED:
+            st.update(guide_hist=np.zeros((c.n_cells, 256), np.float32), guide_cdf=W.random_guide_cdf(c.n_cells, 33))
+        c.set_state(stream=stream, **st)
+        r = c.render_iteration(img, seed=6, iteration=3, mode=mars.MARS_MODE_MARS, profile=profile, stream=stream)
+        torch.cuda.synchronize()
+        out.append((img.cpu().numpy().copy(), r, c.get_state(stream=stream)))
+    return out
+
+
+def _same(a, b):
+    (ia, ra, ga), (ib, rb, gb) = a, b
+    assert np.array_equal(ia, ib)
+    for k in KEYS:
+        assert ra[k] == rb[k], k
+    assert np.array_equal(ga["pixel_rays"], gb["pixel_rays"])
+    np.testing.assert_allclose(ra["mean_beta"], rb["mean_beta"], rtol=1e-9)
+    # float32 sums of runs of equal cells in a warp, in another grouping: 31 additions of 2^-24 each
+    np.testing.assert_allclose(ga["stats"], gb["stats"], rtol=2e-6, atol=1e-9)
+    if "guide_hist" in ga:
+        np.testing.assert_allclose(ga["guide_hist"], gb["guide_hist"], rtol=1e-4, atol=1e-6)
+
+
+# from the first wave on: pixel counts at the edges of a root group and of a block's
+# rays, more pixels than the blocks' targets hold, every technique set and depth limit
+@pytest.mark.parametrize("w,h,D,tech", [(1, 1, 10, TECH3), (7, 1, 3, TECH3), (8, 1, 3, 3), (9, 1, 4, 5), (131, 1, 2, TECH3),
+                                        (64, 48, 1, 1), (97, 61, 10, TECH3), (256, 256, 5, 3), (255, 257, 4, TECH3)])
+def test_whole_path_trees_equal_the_wave_kernels(mars, w, h, D, tech):
+    a, b = _pair(mars, w, h, D, tech, 0.1, 0.6)
+    assert a[1]["wave_launches"] == D and b[1]["wave_launches"] == 0
+    _same(a, b)
+
+
+# from a deeper wave on: images of more than 2^16 pixels, in one and two lanes
+@pytest.mark.parametrize("w,h,lanes", [(300, 260, 1), (500, 300, 1), (500, 300, 2)])
+def test_deep_waves_equal_the_wave_kernels(mars, w, h, lanes):
+    a, b = _pair(mars, w, h, 8, TECH3, 0.05, 0.25, lanes=lanes)
+    assert a[1]["wave_launches"] == 8 and 0 < b[1]["wave_launches"] < 8 * b[1]["tiles"]
+    _same(a, b)
+
+
+def test_slices_that_overflow_are_rendered_by_the_wave_kernels(mars):
+    """A few pixels that split heavily in an arena whose average slice is ample:
+    the tile is rendered again by the wave kernels and gives the same image."""
+    import torch
+    cfg = W.config_box(64, 64)
+    q_rr, q_s, valid = W.random_count_fields(cfg.n_cells, seed=41, lo=0.2, hi=0.5)
+    est = np.full((cfg.scene.n_pixels, 3), 0.5, np.float32)
+    est[2000:2004] = 2e-3
+    out = []
+    for cap in (0, 45000):
+        scene = mars.Scene(cfg.scene)
+        c = mars.Cache(scene, cfg.grid_n, cfg.techniques, cfg.max_depth, arena_capacity=cap)
+        c.set_state(q_rr=q_rr, q_s=q_s, valid=valid, pixel_estimate=est, has_estimate=True, n_iterations=1)
+        img = torch.zeros(3 * cfg.scene.n_pixels, dtype=torch.float32, device="cuda")
+        r = c.render_iteration(img, seed=2, iteration=1, mode=mars.MARS_MODE_MARS, profile=cap == 0)
+        torch.cuda.synchronize()
+        out.append((img.cpu().numpy().copy(), r, c.get_state()))
+    assert out[1][1]["retries"] > 0
+    assert np.array_equal(out[0][0], out[1][0]) and out[0][1]["rays"] == out[1][1]["rays"]
+    np.testing.assert_allclose(out[0][2]["stats"], out[1][2]["stats"], rtol=2e-6, atol=1e-9)
