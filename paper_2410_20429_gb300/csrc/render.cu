@@ -53,69 +53,83 @@ __global__ void k_tile_init(DevCounters* ctr, const IterArgs* __restrict__ itp) 
   }
 }
 
+// One warp, lane d - 1 for depth wave d: the wave's counters are loaded side by
+// side (one thread that added them up took a round trip to memory after another,
+// 7 us at D = 12).
 __global__ void k_tile_finish(DevCounters* ctr, unsigned int* tile_status, const IterArgs* __restrict__ itp, int D) {
-  if (threadIdx.x != 0) return;
-  const int slot = itp->tile_slot;
-  unsigned long long dem = 0;
-  for (int d = 1; d <= D; ++d) {
-    const unsigned long long e = ctr->base[d] + ctr->count[d];
-    dem = e > dem ? e : dem;
+  const int lane = threadIdx.x, d = lane + 1;
+  const bool on = d <= D;
+  const unsigned overflow = ctr->overflow;
+  const unsigned long long base = on ? ctr->base[d] : 0ull, cnt = on ? ctr->count[d] : 0ull;
+  unsigned long long v[5] = {cnt, on ? ctr->scount[d] : 0ull, on ? ctr->slcount[d] : 0ull, on ? ctr->lcount[d] : 0ull,
+                             on ? ctr->vcount[d] : 0ull};
+  const unsigned long long wave_total = on ? ctr->wave_total[d] : 0ull;
+  unsigned long long dem = base + cnt;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const unsigned long long o = __shfl_xor_sync(FULL, dem, off);
+    dem = o > dem ? o : dem;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) v[k] += __shfl_xor_sync(FULL, v[k], off);
   }
+  if (!overflow && on) ctr->wave_total[d] = wave_total + cnt;
+  if (lane != 0) return;
   ctr->demand = dem;
-  if (!ctr->overflow) {
-    unsigned long long tot = 0, sh = 0, sl = 0, lc = 0, lv = 0;
-    for (int d = 1; d <= D; ++d) {
-      tot += ctr->count[d];
-      sh += ctr->scount[d];
-      sl += ctr->slcount[d];
-      lc += ctr->lcount[d];
-      lv += ctr->vcount[d];
-      ctr->wave_total[d] += ctr->count[d];
-    }
-    ctr->entries += tot;
-    ctr->shadow_entries += sh;
-    ctr->shadow_traced += sl;
-    ctr->light_entries += lc;
-    ctr->light_vertex_entries += lv;
+  if (!overflow) {
+    // fire-and-forget additions; nobody else writes these while the tile ends
+    atomicAdd(&ctr->entries, v[0]);
+    atomicAdd(&ctr->shadow_entries, v[1]);
+    atomicAdd(&ctr->shadow_traced, v[2]);
+    atomicAdd(&ctr->light_entries, v[3]);
+    atomicAdd(&ctr->light_vertex_entries, v[4]);
   }
-  tile_status[slot] = ctr->overflow;
-  if (ctr->overflow) ctr->any_overflow = 1;
+  tile_status[itp->tile_slot] = overflow;
+  if (overflow) ctr->any_overflow = 1;
 }
 
-// Totals of a second tile lane's counters into the first's (added, then
-// cleared in the source, so that a later merge adds only what came after).
+// Totals of a second tile lane's counters into the first's (added, then cleared
+// in the source, so that a later merge adds only what came after).  One warp; a
+// lane moves the counters of its number, so that they are loaded side by side.
 __global__ void k_merge_lanes(DevCounters* dst, DevCounters* src) {
-  if (threadIdx.x != 0) return;
-  dst->shadow_entries += src->shadow_entries;
-  dst->shadow_traced += src->shadow_traced;
-  dst->rays += src->rays;
-  dst->vertices += src->vertices;
-  dst->est_vertices += src->est_vertices;
-  dst->entries += src->entries;
-  dst->light_entries += src->light_entries;
-  dst->light_vertex_entries += src->light_vertex_entries;
-  dst->light_rays += src->light_rays;
-  dst->conn_rays += src->conn_rays;
-  src->shadow_entries = src->shadow_traced = src->rays = src->vertices = src->est_vertices = src->entries = 0;
-  src->light_entries = src->light_vertex_entries = src->light_rays = src->conn_rays = 0;
-  for (int d = 0; d < MAXD + 2; ++d) {
-    dst->wave_total[d] += src->wave_total[d];
-    src->wave_total[d] = 0;
-  }
-  for (int k = 0; k < 2; ++k)
-    for (int q = 0; q < 4; ++q) {
-      dst->trace_work[k][q] += src->trace_work[k][q];
-      src->trace_work[k][q] = 0;
+  const int lane = threadIdx.x;
+  unsigned long long* const from[] = {&src->shadow_entries, &src->shadow_traced, &src->rays, &src->vertices,
+                                      &src->est_vertices, &src->entries, &src->light_entries,
+                                      &src->light_vertex_entries, &src->light_rays, &src->conn_rays};
+  unsigned long long* const to[] = {&dst->shadow_entries, &dst->shadow_traced, &dst->rays, &dst->vertices,
+                                    &dst->est_vertices, &dst->entries, &dst->light_entries,
+                                    &dst->light_vertex_entries, &dst->light_rays, &dst->conn_rays};
+  constexpr int N = sizeof(from) / sizeof(from[0]);
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+    if (lane == k) {
+      const unsigned long long v = *from[k];
+      *from[k] = 0;
+      atomicAdd(to[k], v);
     }
-  for (int t = 0; t < NT; ++t) {
-    dst->sum_beta[t] += src->sum_beta[t];
-    src->sum_beta[t] = 0.0;
+  if (lane < MAXD + 2) {
+    const unsigned long long v = src->wave_total[lane];
+    src->wave_total[lane] = 0;
+    atomicAdd(&dst->wave_total[lane], v);
   }
-  if (src->any_overflow) dst->any_overflow = 1;
-  src->any_overflow = 0;
-  dst->check_flags |= src->check_flags;
-  src->check_flags = 0;
-  if (src->demand > dst->demand) dst->demand = src->demand;
+  if (lane >= 20 && lane < 28) {
+    const int k = (lane - 20) >> 2, q = (lane - 20) & 3;
+    const unsigned long long v = src->trace_work[k][q];
+    src->trace_work[k][q] = 0;
+    atomicAdd(&dst->trace_work[k][q], v);
+  }
+  if (lane >= 28 && lane < 28 + NT) {
+    const int t = lane - 28;
+    const double v = src->sum_beta[t];
+    src->sum_beta[t] = 0.0;
+    atomicAdd(&dst->sum_beta[t], v);
+  }
+  if (lane == 31) {
+    if (src->any_overflow) dst->any_overflow = 1;
+    src->any_overflow = 0;
+    if (src->check_flags) atomicOr(&dst->check_flags, src->check_flags);
+    src->check_flags = 0;
+    atomicMax(&dst->demand, src->demand);
+  }
 }
 
 template <int MINB>

@@ -376,30 +376,38 @@ __device__ __forceinline__ void image_means(const DevCache& c, double& VI, doubl
   CI = n > 0.0 ? c.img_acc[1] / n : 0.0;
 }
 
-// one warp: V_I and C_I from the slots' sums (and the rejection's subtraction)
+// one warp: V_I and C_I from the slots' sums (and the rejection's subtraction).
+// Every value is loaded before the first is used or written: one round trip to
+// memory instead of one after another.
 __global__ void k_img_final(DevCache c, int npix) {
-  if (c.ctr->any_overflow) return;
-  double v64 = c.ctr->img_part[threadIdx.x][3];
-  float v32 = c.ctr->img_part32[threadIdx.x][3];
+  DevCounters* ctr = c.ctr;
+  const unsigned overflow = ctr->any_overflow;
+  double v64 = ctr->img_part[threadIdx.x][3];
+  float v32 = ctr->img_part32[threadIdx.x][3];
+  double sum64 = ctr->vi_sum;
+  float sum32 = ctr->vi_sum32;
+  const int dropped = ctr->vi_dropped;
+  const unsigned long long rays = ctr->rays;
+  const double a0 = c.img_acc[0], a1 = c.img_acc[1], a2 = c.img_acc[2];
+  if (overflow) return;
   for (int off = 16; off > 0; off >>= 1) {
     v64 += __shfl_xor_sync(0xffffffffu, v64, off);
     v32 += __shfl_xor_sync(0xffffffffu, v32, off);
   }
   if (threadIdx.x != 0) return;
-  c.ctr->vi_sum += v64;
-  c.ctr->vi_sum32 += v32;
-  const int kept = npix - c.ctr->vi_dropped;  // V_I: the mean over the pixels that were kept
-  if (c.stats32) {
-    c.ctr->VI = (double)(c.ctr->vi_sum32 / (3.0f * (float)kept));
-    c.ctr->CI = (double)((float)c.ctr->rays / (float)npix);
-  } else {
-    c.ctr->VI = c.ctr->vi_sum / (3.0 * (double)kept);
-    c.ctr->CI = (double)c.ctr->rays / (double)npix;
-  }
+  sum64 += v64;
+  sum32 += v32;
+  const int kept = npix - dropped;  // V_I: the mean over the pixels that were kept
+  const double VI = c.stats32 ? (double)(sum32 / (3.0f * (float)kept)) : sum64 / (3.0 * (double)kept);
+  const double CI = c.stats32 ? (double)((float)rays / (float)npix) : (double)rays / (double)npix;
+  ctr->vi_sum = sum64;
+  ctr->vi_sum32 = sum32;
+  ctr->VI = VI;
+  ctr->CI = CI;
   // a training iteration of several such iterations: the update averages them
-  c.img_acc[0] += c.ctr->VI;
-  c.img_acc[1] += c.ctr->CI;
-  c.img_acc[2] += 1.0;
+  c.img_acc[0] = a0 + VI;
+  c.img_acc[1] = a1 + CI;
+  c.img_acc[2] = a2 + 1.0;
 }
 
 __global__ void k_update_counts(DevCache c) {
