@@ -616,16 +616,9 @@ mars_status cache_create_impl(const mars_scene* s, const mars_cache_desc* d, cud
   cudaMemsetAsync(c->d_img, 0, sizeof(float4) * pixels, st);
   cudaMemsetAsync(c->d_ctr, 0, sizeof(DevCounters) * mars_cache::kMaxLanes, st);
   cudaMemsetAsync(c->d_tile_status, 0, sizeof(unsigned int) * c->max_tiles, st);
-  {
-    std::vector<float> cdf((size_t)GUIDE_BINS * gcells);
-    for (int64_t k = 0; k < gcells; ++k)
-      for (int b = 0; b < GUIDE_BINS; ++b) cdf[k * GUIDE_BINS + b] = (float)((double)(b + 1) / GUIDE_BINS);
-    std::vector<float4> one((size_t)pixels, make_float4(1.f, 1.f, 1.f, 0.f));
-    if ((e = cudaMemcpyAsync(c->d_cdf, cdf.data(), sizeof(float) * cdf.size(), cudaMemcpyHostToDevice, st)) ||
-        (e = cudaMemcpyAsync(c->d_est, one.data(), sizeof(float4) * one.size(), cudaMemcpyHostToDevice, st)))
-      return cleanup(e, "cache init");
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cleanup(e, "cache init");
-  }
+  if ((e = launch_cache_fill(c->d_cdf, gcells, c->d_est, pixels, s->num_sms, st)) != cudaSuccess ||
+      (e = cudaStreamSynchronize(st)) != cudaSuccess)
+    return cleanup(e, "cache init");
   c->dc.grid_n = d->grid_n;
   c->dc.n_cells = (int)cells;
   c->dc.techniques = d->techniques;

@@ -315,6 +315,8 @@ cudaError_t launch_combined_out(const DevCache& c, int npix, float* out, cudaStr
 cudaError_t launch_image_copy(const DevCache& c, int npix, float* out, cudaStream_t st);
 // the iteration image of pixels [p0, p1) only, packed rgb, into out (device; the whole frame's layout)
 cudaError_t launch_image_copy_range(const DevCache& c, int p0, int p1, float* out, cudaStream_t st);
+// uniform guide CDFs and unit pixel estimates of a new cache
+cudaError_t launch_cache_fill(float* cdf, int64_t cells, float4* est, int64_t pixels, int num_sms, cudaStream_t st);
 cudaError_t launch_update(const DevCache& c, int num_sms, cudaStream_t st);
 // octree refinement after an update (stats.cu): leaf_samples must run before
 // launch_update (which zeroes the statistics), refine after it

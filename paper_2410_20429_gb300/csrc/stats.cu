@@ -688,7 +688,28 @@ __global__ void k_octree_inherit(DevCache c) {
   }
 }
 
+// A new cache's guide CDFs (uniform: bin b at (b + 1) / 256, exact in float32)
+// and pixel estimates (1), four floats a thread.  Filled on the host and copied
+// from pageable memory they took most of a small request's set-up (cache creation, 256^2, 24^3
+// cells: 3.2 -> 0.64 ms).
+__global__ void k_cache_fill(float4* __restrict__ cdf, size_t n_cdf, float4* __restrict__ est, size_t n_est) {
+  const size_t stride = gridDim.x * (size_t)blockDim.x;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n_cdf; i += stride) {
+    const float b = (float)(4 * (i % (GUIDE_BINS / 4)));
+    constexpr float w = 1.0f / GUIDE_BINS;
+    cdf[i] = make_float4((b + 1.0f) * w, (b + 2.0f) * w, (b + 3.0f) * w, (b + 4.0f) * w);
+  }
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n_est; i += stride)
+    est[i] = make_float4(1.f, 1.f, 1.f, 0.f);
+}
+
 }  // namespace
+
+cudaError_t launch_cache_fill(float* cdf, int64_t cells, float4* est, int64_t pixels, int num_sms, cudaStream_t st) {
+  k_cache_fill<<<4 * num_sms, 256, 0, st>>>(reinterpret_cast<float4*>(cdf), (size_t)cells * (GUIDE_BINS / 4), est,
+                                            (size_t)pixels);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_leaf_samples(const DevCache& c, cudaStream_t st) {
   k_leaf_samples<<<(c.n_cells + 255) / 256, 256, 0, st>>>(c);
