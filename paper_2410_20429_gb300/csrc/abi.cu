@@ -834,7 +834,8 @@ static DevCache lane_cache(const mars_cache* c, int l) {
 }
 
 // The depth from which on an iteration of `pixels` pixels a lane, with a ray arena
-// of `cap` slots a lane, runs in k_tail (0: nowhere): the first wave of at most
+// of `cap` slots a lane, runs in k_tail (with light connections: joins its waves'
+// side kernels, which needs no room); 0: nowhere.  The first wave of at most
 // kTailRays rays, its size and those of the deeper waves taken from the last
 // iteration's rays per pixel (the first wave's is known), if what the waves
 // before leave of the arena holds the rest with tail_margin to spare -- a block's
@@ -846,7 +847,8 @@ static DevCache lane_cache(const mars_cache* c, int l) {
 // k_tail 0.844, 1.165 and 2.63.  Larger waves fill the GPU by themselves.
 constexpr double kTailRays = 65536.0;
 static int tail_depth(const mars_cache* c, int64_t pixels, uint64_t cap) {
-  if (c->tail_blocks <= 0 || cap > (1ull << 31)) return 0;
+  const bool light = (c->techniques & MARS_TECH_LIGHT) != 0;
+  if (!light && (c->tail_blocks <= 0 || cap > (1ull << 31))) return 0;
   const double scale = c->last_pixels > 0 ? (double)pixels / (double)c->last_pixels : 0.0;
   double before = 0.0, after = 0.0;
   for (int d = 1; d <= c->max_depth; ++d) after += scale * (double)c->last_wave[d];
@@ -856,7 +858,7 @@ static int tail_depth(const mars_cache* c, int64_t pixels, uint64_t cap) {
     before += wave;
     after -= scale * (double)c->last_wave[k];
     const double least = k == 1 ? 1.5 * (c->max_depth - 1) * (double)pixels : 0.0;
-    if (wave <= kTailRays && (double)cap - before >= std::max(c->tail_margin * after, least)) return k;
+    if (wave <= kTailRays && (light || (double)cap - before >= std::max(c->tail_margin * after, least))) return k;
   }
   return 0;
 }
@@ -1117,7 +1119,7 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
       return poison(c, e, "render launch");
     }
     launches += (uint32_t)(tiles.size() * tile_launches(D, c->techniques, tail)) + (uint32_t)(nl - 1);
-    wave_launches += (uint32_t)(tiles.size() * (tail > 0 ? tail - 1 : D));
+    wave_launches += (uint32_t)(tiles.size() * (tail > 0 && !(c->techniques & MARS_TECH_LIGHT) ? tail - 1 : D));
     launches += p->update_estimate ? 3 + (p->vi_drop_brightest > 0 ? 2 : 0) + (p->combine ? 1 : 0)
                                    : (dev_out ? 1 : 0);
     used += (uint32_t)tiles.size();

@@ -84,18 +84,25 @@ __device__ __forceinline__ unsigned long long vertex_base(const DevCounters* ctr
   return b;
 }
 
-// One thread per light connection sample of wave d (a warp-uniform loop: the
-// light vertex slots are allocated per warp): its light subpath, then the
-// per-vertex terms the connections' weights need, written to the light vertex
-// region; LR = (first vertex slot, m, pN, cost).
+// light connection samples of the waves d..d1, which lie one wave after the other
+__device__ __forceinline__ unsigned long long light_samples(const DevCounters* ctr, int d, int d1) {
+  unsigned long long n = 0;
+  for (int e = d; e <= d1; ++e) n += ctr->lcount[e];
+  return n;
+}
+
+// One thread per light connection sample of the waves d..d1 (a warp-uniform loop:
+// the light vertex slots are allocated per warp, all from wave d's count): its
+// light subpath, then the per-vertex terms the connections' weights need,
+// written to the light vertex region; LR = (first vertex slot, m, pN, cost).
 template <int MINB>
 __global__ void __launch_bounds__(MAX_LIGHT_THREADS, MINB) k_light_path(const DevScene s, const DevCache c,
                                                                const Arena a, const IterArgs* __restrict__ itp,
-                                                               const int d) {
+                                                               const int d, const int d1) {
   const IterArgs it = *itp;
   DevCounters* ctr = c.ctr;
   if (ctr->overflow) return;  // the tile is re-rendered
-  const unsigned long long lb = ctr->lbase[d], lc = ctr->lcount[d];
+  const unsigned long long lb = ctr->lbase[d], lc = light_samples(ctr, d, d1);
   const unsigned long long n = lb >= a.lcap ? 0ull : (lc < a.lcap - lb ? lc : a.lcap - lb);
   const unsigned long long vb = vertex_base(ctr, d);
   const Rng rng{it.seed, it.job, it.iteration};
@@ -239,7 +246,7 @@ __global__ void __launch_bounds__(MAX_LIGHT_THREADS, MINB) k_light_path(const De
   if (lane == 0 && n_rays) atomicAdd(&ctr->light_rays, n_rays);
 }
 
-// One thread per light vertex y_k of wave d's samples: the connection x_i --
+// One thread per light vertex y_k of those samples: the connection x_i --
 // y_k, its contribution alpha_k f_y f_x / d^2, its balance weight over every
 // strategy of the full path, and a shadow ray; LC = the weighted contribution
 // if visible, else zero.
@@ -400,16 +407,16 @@ __global__ void __launch_bounds__(MAX_LIGHT_THREADS, MINB) k_light_connect(const
 int light_variants() { return 3; }
 
 cudaError_t launch_light(const DevScene& s, const DevCache& c, const Arena& a, const IterArgs* it, int variant,
-                         int grid, int threads, int d, cudaStream_t st) {
+                         int grid, int threads, int d, int d1, cudaStream_t st) {
   if (threads > MAX_LIGHT_THREADS) threads = MAX_LIGHT_THREADS;
   if (variant == 2) {
-    k_light_path<3><<<grid, threads, 0, st>>>(s, c, a, it, d);
+    k_light_path<3><<<grid, threads, 0, st>>>(s, c, a, it, d, d1);
     k_light_connect<3><<<grid, threads, 0, st>>>(s, c, a, it, d);
   } else if (variant == 1) {
-    k_light_path<2><<<grid, threads, 0, st>>>(s, c, a, it, d);
+    k_light_path<2><<<grid, threads, 0, st>>>(s, c, a, it, d, d1);
     k_light_connect<2><<<grid, threads, 0, st>>>(s, c, a, it, d);
   } else {
-    k_light_path<1><<<grid, threads, 0, st>>>(s, c, a, it, d);
+    k_light_path<1><<<grid, threads, 0, st>>>(s, c, a, it, d, d1);
     k_light_connect<1><<<grid, threads, 0, st>>>(s, c, a, it, d);
   }
   return cudaGetLastError();

@@ -274,15 +274,16 @@ struct WaveLaunch {
   int grid[WAVE_KERNELS];                  // persistent grid: SMs x resident blocks
 };
 
-// the light connection kernel of wave d (bdpt.cu)
+// the light connection kernels of the waves d..d1 (bdpt.cu)
 cudaError_t launch_light(const DevScene& s, const DevCache& c, const Arena& a, const IterArgs* it, int variant,
-                         int grid, int threads, int d, cudaStream_t st);
+                         int grid, int threads, int d, int d1, cudaStream_t st);
 int light_variants();
 
 // launch wrappers (render.cu)
 // it: device pointer to the tile's arguments
 // tail: the waves from this depth on run in k_tail, with tail_blocks blocks (0:
-// every wave in the wave kernels; always 0 with light connections)
+// every wave in the wave kernels); with light connections, the depth from which
+// on several waves share a launch of the side streams' kernels
 // side2: the light connection kernels' stream (light connections only; null:
 // they run on side); sync: D + 2 events
 cudaError_t launch_tile(const DevScene& s, const DevCache& c, const Arena& a, const IterArgs* it,

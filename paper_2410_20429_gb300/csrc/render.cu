@@ -207,19 +207,22 @@ __global__ void __launch_bounds__(MAX_WAVE_THREADS, MINB) k_shade(const DevScene
 }
 
 // ----------------------------------------------------------------- shadow
-// the listed shadow rays of wave d: SH0, SH1[sbase, sbase + slcount) (at most
-// scount of them), each with the slot of its sample's value
+// the listed shadow rays of the waves d..d1: SH0, SH1[sbase, sbase + slcount) of
+// each (at most scount of them), each with the slot of its sample's value
 template <int MINB>
 __global__ void __launch_bounds__(MAX_WAVE_THREADS, MINB) k_shadow(const DevScene s, const DevCache c, const Arena a,
-                                                           const int d) {
+                                                           const int d, const int d1) {
   DevCounters* ctr = c.ctr;
   if (ctr->overflow) return;
   extern __shared__ RayStage ray_stage[];
-  const unsigned long long sb = ctr->sbase[d], sl = ctr->slcount[d];
-  const unsigned long long n = sl < a.scap - sb ? sl : a.scap - sb;
   TraceWork tw;
-  shadow_hits(s, c, a, sb, (unsigned)n, &ctr->shadow_next[d], (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-              (gridDim.x * blockDim.x) >> 5, ray_stage + (threadIdx.x >> 5), tw);
+  for (int e = d; e <= d1; ++e) {
+    const unsigned long long sb = ctr->sbase[e], sl = ctr->slcount[e];
+    const unsigned long long n = sl < a.scap - sb ? sl : a.scap - sb;
+    if (n > 0)
+      shadow_hits(s, c, a, sb, (unsigned)n, &ctr->shadow_next[e], (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                  (gridDim.x * blockDim.x) >> 5, ray_stage + (threadIdx.x >> 5), tw);
+  }
   flush_work(tw, ctr->trace_work[1], ctr);
 }
 
@@ -251,7 +254,7 @@ size_t shade_smem(int threads) { return (size_t)(threads / 32) * sizeof(ShadeWar
 // 3.62 -> 2.97, 524k at 2048^2 13.4 -> 11.7).  k_reverse keeps its registers
 // (capped at 80, 512^2 warm-up 0.86 -> 0.91 ms).
 using TraceFn = void (*)(const DevScene, const DevCache, const Arena, const IterArgs*, const int);
-using ShadowFn = void (*)(const DevScene, const DevCache, const Arena, const int);
+using ShadowFn = void (*)(const DevScene, const DevCache, const Arena, const int, const int);
 TraceFn trace_fn(int v) { return v == 2 ? k_trace<6> : k_trace<4>; }
 TraceFn shade_fn(int v, bool bd = false) {
   if (bd) return v == 2 ? k_shade<4, true> : k_shade<3, true>;
@@ -292,6 +295,19 @@ cudaError_t wave_occupancy(const int threads[WAVE_KERNELS], const int variant[WA
 
 bool wave_threads_ok(int threads) { return threads >= 32 && threads <= MAX_WAVE_THREADS && threads % 32 == 0; }
 
+// Whether the shadow and light connection kernels launched after wave d's shading
+// take the waves up to d that earlier launches left.  With light connections the
+// waves from `tail` on, all small, go three at a time: a launch of the light
+// kernels lasts as long as its longest subpath (up to five traversals one after
+// the other, 150 us and more) however few samples a wave has, and the launches of
+// one stream follow one another.  Heightfield of 131k triangles, wave by wave -> in
+// threes: 128^2 1.15 -> 0.83 ms, 256^2 1.45 -> 1.12, 512^2 2.08 -> 1.76, 1024^2 4.41 ->
+// 4.23; in twos 0.85, 1.12, 1.83 and 4.22, all in one 0.98, 1.28, 1.84 and 4.29 (they
+// then start late).
+static bool side_batch_ends(int d, int D, int tail) {
+  return tail <= 0 || d < tail || (d - tail) % 3 == 2 || d == D - 2 || d == D - 1;
+}
+
 cudaError_t launch_tile(const DevScene& s, const DevCache& c, const Arena& a, const IterArgs* it, const WaveLaunch& L,
                         int64_t tile_pixels, int tail, int tail_blocks, cudaStream_t st, cudaStream_t side, cudaStream_t side2, const cudaEvent_t* sync,
                         cudaEvent_t* ev) {
@@ -324,31 +340,35 @@ cudaError_t launch_tile(const DevScene& s, const DevCache& c, const Arena& a, co
   if (ev) cudaEventRecord(ev[0], st);
   cudaStream_t lside = side2 ? side2 : side;
   bool any_shadow = false, any_light = false;
-  const int last = tail > 0 ? tail - 1 : D;  // the deepest wave of the wave kernels
+  const int last = !bd && tail > 0 ? tail - 1 : D;  // the deepest wave of the wave kernels
+  int first = 1;
   for (int d = 1; d <= last; ++d) {
     trace_fn(L.variant[WK_TRACE])<<<G(WK_TRACE, d), tT, trace_smem(tT), st>>>(s, c, a, it, d);
     if (ev) cudaEventRecord(ev[2 * (d - 1) + 1], st);
     shade_fn(L.variant[WK_SHADE], bd)<<<G(WK_SHADE, d), tS, smS, st>>>(s, c, a, it, d);
     if (ev) cudaEventRecord(ev[2 * (d - 1) + 2], st);
-    const bool shadow = d <= D - 1 && nee, light = bd && d <= D - 2;
+    if (!side_batch_ends(d, D, bd ? tail : 0)) continue;
+    // the side kernels of the waves first..d
+    const bool shadow = first <= D - 1 && nee, light = bd && first <= D - 2;
     if (shadow || light) cudaEventRecord(sync[d - 1], st);
     if (shadow) {
       cudaStreamWaitEvent(side, sync[d - 1], 0);
       any_shadow = true;
       if (ev) cudaEventRecord(ev[2 * D + 2 * (d - 1) + 1], side);
-      shadow_fn(L.variant[WK_SHADOW])<<<G(WK_SHADOW, d), tH, trace_smem(tH), side>>>(s, c, a, d);
+      shadow_fn(L.variant[WK_SHADOW])<<<G(WK_SHADOW, d), tH, trace_smem(tH), side>>>(s, c, a, first, std::min(d, D - 1));
       if (ev) cudaEventRecord(ev[2 * D + 2 * (d - 1) + 2], side);
     }
     if (light) {
       if (lside != side || !shadow) cudaStreamWaitEvent(lside, sync[d - 1], 0);
       any_light = true;
       if (ev) cudaEventRecord(ev[5 * D + 2 + 2 * (d - 1)], lside);
-      cudaError_t e = launch_light(s, c, a, it, L.variant[WK_SHADOW], G(WK_SHADOW, d), tH, d, lside);
+      cudaError_t e = launch_light(s, c, a, it, L.variant[WK_SHADOW], G(WK_SHADOW, d), tH, first, std::min(d, D - 2), lside);
       if (e != cudaSuccess) return e;
       if (ev) cudaEventRecord(ev[5 * D + 2 + 2 * (d - 1) + 1], lside);
     }
+    first = d + 1;
   }
-  if (tail > 0) launch_tail(s, c, a, it, tail, tail_blocks, st);
+  if (!bd && tail > 0) launch_tail(s, c, a, it, tail, tail_blocks, st);
   if (any_shadow) {
     cudaEventRecord(sync[D], side);
     cudaStreamWaitEvent(st, sync[D], 0);
@@ -361,7 +381,7 @@ cudaError_t launch_tile(const DevScene& s, const DevCache& c, const Arena& a, co
     cudaStreamWaitEvent(st, sync[D], 0);
   }
   if (ev) cudaEventRecord(ev[5 * D + 1], st);
-  if (tail > 0) launch_tail_reverse(s, c, a, it, tail, tail_blocks, st);
+  if (!bd && tail > 0) launch_tail_reverse(s, c, a, it, tail, tail_blocks, st);
   for (int d = last; d >= 1; --d) {
     reverse_fn(L.variant[WK_REVERSE], bd)<<<G(WK_REVERSE, d), tR, 0, st>>>(s, c, a, it, d);
     if (ev) cudaEventRecord(ev[4 * D + (D - d + 1)], st);
@@ -376,10 +396,16 @@ cudaError_t launch_merge_lanes(DevCounters* dst, DevCounters* src, cudaStream_t 
 }
 
 int tile_launches(int max_depth, int techniques, int tail) {
-  if (tail > 0) return 4 + 3 * (tail - 1) + ((techniques & MARS_TECH_NEE) ? tail - 1 : 0);
-  // light connections: a light-subpath and a connection kernel per wave of depth <= D - 2
-  return 2 + 2 * max_depth + max_depth + ((techniques & MARS_TECH_NEE) ? max_depth - 1 : 0) +
-         ((techniques & MARS_TECH_LIGHT) && max_depth > 2 ? 2 * (max_depth - 2) : 0);
+  const bool nee = (techniques & MARS_TECH_NEE) != 0, bd = (techniques & MARS_TECH_LIGHT) != 0;
+  const int D = max_depth, last = !bd && tail > 0 ? tail - 1 : D;
+  int n = 2 + 3 * last + (last < D ? 2 : 0);  // begin and end, trace, shade, reverse, the tail kernels
+  for (int d = 1, first = 1; d <= last; ++d) {
+    if (!side_batch_ends(d, D, bd ? tail : 0)) continue;
+    if (nee && first <= D - 1) ++n;
+    if (bd && first <= D - 2) n += 2;  // light subpaths, connections
+    first = d + 1;
+  }
+  return n;
 }
 
 }  // namespace mars

@@ -100,3 +100,14 @@ def test_slices_that_overflow_are_rendered_by_the_wave_kernels(mars):
     assert out[1][1]["retries"] > 0
     assert np.array_equal(out[0][0], out[1][0]) and out[0][1]["rays"] == out[1][1]["rays"]
     np.testing.assert_allclose(out[0][2]["stats"], out[1][2]["stats"], rtol=2e-6, atol=1e-9)
+
+
+# with light connections the small waves share launches of the shadow and light
+# kernels: at every remainder of the batches and the depth limits of both techniques
+@pytest.mark.parametrize("D", [1, 2, 3, 4, 5, 6, 7, 9])
+def test_joined_side_kernels_equal_the_waves_own(mars, D):
+    a, b = _pair(mars, 61, 47, D, W.TECH_BSDF | W.TECH_NEE | W.TECH_LIGHT, 0.3, 0.9)
+    _same(a, b)
+    assert b[1]["launches"] <= a[1]["launches"]
+    for k in ("light_rays", "connection_rays", "light_samples"):
+        assert a[1][k] == b[1][k], k
