@@ -133,7 +133,8 @@ def sm_max_mhz():
 OPS_NODE, OPS_QUAD, OPS_SPHERE, OPS_TRI = 50, 67, 25, 45
 
 
-KERNEL_SOURCES = ["paper_2410_20429_gb300/csrc/render.cu", "paper_2410_20429_gb300/csrc/device.cuh",
+KERNEL_SOURCES = ["paper_2410_20429_gb300/csrc/render.cu", "paper_2410_20429_gb300/csrc/wave.cuh",
+                  "paper_2410_20429_gb300/csrc/device.cuh",
                   "paper_2410_20429_gb300/csrc/internal.h", "paper_2410_20429_gb300/build.py"]
 TRAFFIC_FILE = "profiles/dram_traffic_wave_kernels_guided_room_256.txt"
 SERVE_MULTIPLICITY = 16.0   # the server's path multiplicity cap for served jobs (csrc/server.cu)

@@ -236,7 +236,7 @@ typedef struct {
   float wave_ms[4][16];       /* profile = 1: device ms of trace, shade, shadow, reverse per depth wave d (index d - 1) */
   uint64_t wave_rays[16];     /* rays held by depth wave d (index d - 1), all tiles */
   uint64_t trace_work[2][4];  /* closest-hit [0] and shadow [1] traversal: BVH node visits
-                                 (two box tests each), quad, sphere and triangle tests */
+                                 (of two box tests; a 4-wide node counts as two), quad, sphere and triangle tests */
   uint32_t check_flags;       /* MARS_CHECK_* bits of the index checks that failed (always 0
                                  in the regular library; see below) */
   uint32_t reserved;
@@ -313,13 +313,13 @@ typedef struct {
 } mars_cache_info;
 
 /* ---- scene ------------------------------------------------------------
- * Copies the description to the device, builds the closest-hit hierarchy
+ * Copies the description to the device, builds the hierarchy
  * selected by desc->bvh -- by default (MARS_BVH_SAH) a top-down surface-area
  * heuristic build on the host CPU (binned above 64 primitives, exact sweeps
  * below; about 0.1 s for 131k triangles, 0.4 s for 524k), with MARS_BVH_LBVH a
  * linear BVH built on the device (Morton codes, sort, Karras hierarchy,
  * bottom-up bounds); either is validated on the host and collapsed into the
- * 4-wide hierarchy of the shadow rays -- and the light-selection table
+ * 4-wide hierarchy that every ray walks -- and the light-selection table
  * (probability proportional to area x mean radiance).  Results do not depend
  * on the hierarchy.  Synchronises `stream` before returning.  Errors: INVALID_ARG (no primitives, bad sizes,
  * material index out of range, emitting sphere/triangle), OOM, CUDA. */
