@@ -1177,10 +1177,12 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
     for (size_t t = 0; t < tiles.size(); ++t) {
       if (!c->h_tile_status[t]) continue;
       const int64_t a = tiles[t].first, b = tiles[t].second;
-      if (b - a <= 1)
+      if (b - a <= 1 && !(tail > 0 && !(c->techniques & MARS_TECH_LIGHT)))
         return set_error(MARS_ERR_OOM, "one pixel's path tree needs more than the arena's %llu rays",
                          (unsigned long long)(c->arena.cap / (uint64_t)std::max(1, nl)));
-      const int64_t parts = std::min<int64_t>(k, b - a);
+      // a tile that k_tail's slices were too small for goes to the wave kernels whole,
+      // which have all of the arena for it
+      const int64_t parts = tail > 0 && !(c->techniques & MARS_TECH_LIGHT) ? 1 : std::min<int64_t>(k, b - a);
       for (int64_t j = 0; j < parts; ++j) again.emplace_back(a + (b - a) * j / parts, a + (b - a) * (j + 1) / parts);
     }
     if (again.empty()) break;

@@ -111,3 +111,20 @@ def test_joined_side_kernels_equal_the_waves_own(mars, D):
     assert b[1]["launches"] <= a[1]["launches"]
     for k in ("light_rays", "connection_rays", "light_samples"):
         assert a[1][k] == b[1][k], k
+
+
+def test_a_tile_whose_slices_overflow_is_rendered_again_whole(mars):
+    """The arena holds the tile with room to spare, but not the subtrees of a few
+    pixels in their blocks' slices: one more attempt, of the same tile."""
+    import torch
+    cfg = W.config_box(64, 64)
+    q_rr, q_s, valid = W.random_count_fields(cfg.n_cells, seed=41, lo=0.2, hi=0.5)
+    est = np.full((cfg.scene.n_pixels, 3), 0.5, np.float32)
+    est[2000:2004] = 2e-3
+    scene = mars.Scene(cfg.scene)
+    c = mars.Cache(scene, cfg.grid_n, cfg.techniques, cfg.max_depth, arena_capacity=45000)
+    c.set_state(q_rr=q_rr, q_s=q_s, valid=valid, pixel_estimate=est, has_estimate=True, n_iterations=1)
+    img = torch.zeros(3 * cfg.scene.n_pixels, dtype=torch.float32, device="cuda")
+    r = c.render_iteration(img, seed=2, iteration=1, mode=mars.MARS_MODE_MARS)
+    assert r["wave_entries"] < 45000
+    assert r["retries"] == 1 and r["tiles"] == 2
