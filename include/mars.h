@@ -225,7 +225,7 @@ typedef struct {
   double mean_beta[3];        /* mean beta per technique slot over estimator vertices */
   uint32_t tiles;             /* pixel tiles used (1 unless the arena overflowed) */
   uint32_t retries;           /* tiles re-rendered after an overflow */
-  uint64_t arena_demand;      /* rays the largest tile needed */
+  uint64_t arena_demand;      /* rays the largest tile needed, all its depths together */
   uint32_t launches;          /* kernels this call launched */
   uint32_t wave_launches;     /* launches of each per-wave kernel (depth waves x tiles) */
   /* device time per kernel kind, summed over waves and tiles (profile = 1) */

@@ -60,21 +60,20 @@ __global__ void k_tile_finish(DevCounters* ctr, unsigned int* tile_status, const
   const int lane = threadIdx.x, d = lane + 1;
   const bool on = d <= D;
   const unsigned overflow = ctr->overflow;
-  const unsigned long long base = on ? ctr->base[d] : 0ull, cnt = on ? ctr->count[d] : 0ull;
+  const unsigned long long cnt = on ? ctr->count[d] : 0ull;
   unsigned long long v[5] = {cnt, on ? ctr->scount[d] : 0ull, on ? ctr->slcount[d] : 0ull, on ? ctr->lcount[d] : 0ull,
                              on ? ctr->vcount[d] : 0ull};
   const unsigned long long wave_total = on ? ctr->wave_total[d] : 0ull;
-  unsigned long long dem = base + cnt;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
-    const unsigned long long o = __shfl_xor_sync(FULL, dem, off);
-    dem = o > dem ? o : dem;
 #pragma unroll
     for (int k = 0; k < 5; ++k) v[k] += __shfl_xor_sync(FULL, v[k], off);
   }
   if (!overflow && on) ctr->wave_total[d] = wave_total + cnt;
   if (lane != 0) return;
-  ctr->demand = dem;
+  // every ray of the tile, drawn by whichever kernels: the waves lie one after the
+  // other, and k_tail counts its rays by depth without placing its waves
+  ctr->demand = v[0];
   if (!overflow) {
     // fire-and-forget additions; nobody else writes these while the tile ends
     atomicAdd(&ctr->entries, v[0]);

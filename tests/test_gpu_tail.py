@@ -128,3 +128,13 @@ def test_a_tile_whose_slices_overflow_is_rendered_again_whole(mars):
     r = c.render_iteration(img, seed=2, iteration=1, mode=mars.MARS_MODE_MARS)
     assert r["wave_entries"] < 45000
     assert r["retries"] == 1 and r["tiles"] == 2
+
+
+@pytest.mark.parametrize("w,h,D", [(97, 61, 10), (300, 260, 8)])
+def test_arena_demand_counts_every_depth(mars, w, h, D):
+    """The rays the tile needed, whichever kernels rendered it (from the first
+    wave on, from a deeper one on): all its depths' rays, so that an arena of that
+    many slots holds the tile again."""
+    a, b = _pair(mars, w, h, D, TECH3, 0.1, 0.6, lanes=1)
+    assert a[1]["wave_launches"] > b[1]["wave_launches"]
+    assert b[1]["arena_demand"] == a[1]["arena_demand"] == a[1]["wave_entries"]
