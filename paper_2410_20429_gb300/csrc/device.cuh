@@ -199,10 +199,13 @@ constexpr int STACK = TRAVERSAL_STACK;
 // between an axis's two planes.  o / d is rounded, so the near constant is
 // lowered and the far one raised by 2^-22 of it (four times its rounding
 // error): a box is never left out that exact arithmetic would admit.  A component
-// of d that is zero (or below 1e-20, or not finite) counts as 1e-20: its planes
-// lie at huge distances on the side that tells whether the origin is between
-// them, as the infinities of a division by zero would, without their NaN.  An
-// origin that is not a number meets no box.
+// of d that is zero (or below 1e-20) counts as 1e-20: its planes lie at huge
+// distances on the side that tells whether the origin is between them, as the
+// infinities of a division by zero would, without their NaN; where o / d itself
+// then overflows (|o| above 3e18) the axis leaves the box to the other two.  A ray
+// whose origin or direction is not finite, and one that every axis would leave to
+// the others, meets no box: an unused slot must never be met, for the bound on
+// the stack counts a node's children alone.
 struct SlabRay {
   float ix, iy, iz;           // 1 / d
   float nx, ny, nz;           // near plane constants
@@ -219,8 +222,15 @@ __device__ __forceinline__ SlabRay slab_ray(f3 o, f3 d) {
   constexpr float SLACK = 2.3841858e-7f;   // 2^-22
   const float ex = SLACK * fabsf(ox), ey = SLACK * fabsf(oy), ez = SLACK * fabsf(oz);
   const float inf = __int_as_float(0x7f800000);
-  r.nx = ox == ox ? -ox - ex : inf; r.ny = oy == oy ? -oy - ey : inf; r.nz = oz == oz ? -oz - ez : inf;
-  r.fx = ex - ox; r.fy = ey - oy; r.fz = ez - oz;
+  const bool bx = fabsf(ox) < inf, by = fabsf(oy) < inf, bz = fabsf(oz) < inf;
+  r.nx = bx ? -ox - ex : -inf; r.ny = by ? -oy - ey : -inf; r.nz = bz ? -oz - ez : -inf;
+  r.fx = bx ? ex - ox : inf; r.fy = by ? ey - oy : inf; r.fz = bz ? ez - oz : inf;
+  // x - x is 0 for a finite x only
+  const f3 zo = o - o, zd = d - d;
+  if (!(zo.x + zo.y + zo.z + zd.x + zd.y + zd.z == 0.0f && (bx || by || bz))) {
+    r.nx = r.ny = r.nz = inf;
+    r.fx = r.fy = r.fz = -inf;
+  }
   r.kx = r.ix < 0.0f ? 3 : 0; r.ky = r.iy < 0.0f ? 4 : 1; r.kz = r.iz < 0.0f ? 5 : 2;
   return r;
 }

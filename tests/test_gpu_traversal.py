@@ -85,3 +85,22 @@ def test_hits_and_visibility_of_a_path_tree(mars, orc, w, h, bvh, nested):
     ok = (np.abs(g - o.image) <= 1e-4 * np.abs(o.image) + 1e-7).all(axis=1)
     assert (~ok).sum() <= -(-sc.n_pixels // 500) * (sc.n_pixels >= 500), np.flatnonzero(~ok)[:5]
     assert abs(st["rays"] - o.rays) <= 2e-3 * o.rays and abs(st["vertices"] - o.vertices) <= 2e-3 * o.vertices
+
+
+@pytest.mark.parametrize("part,value", [((0, 1, 2), np.nan), ((0, 1, 2), np.inf), ((1,), -np.inf), ((0,), np.nan),
+                                        ((3, 4, 5), np.nan), ((5,), np.inf)])
+@pytest.mark.parametrize("w,h,lo,hi", [(33, 7, 0.1, 0.6), (97, 61, 0.1, 0.6)])
+def test_rays_that_are_not_finite_meet_nothing(mars, w, h, lo, hi, part, value):
+    """A camera whose origin (0..2) or look-at point (3..5) is not finite: every
+    camera ray visits the root alone and misses."""
+    import torch
+    sc = _lambert_room(w, h, True)
+    sc.camera = sc.camera.copy()
+    sc.camera[list(part)] = value
+    s = mars.Scene(sc)
+    c = mars.Cache(s, 4, W.TECH_BSDF | W.TECH_NEE, 3)
+    for profile in (True, False):
+        img = torch.ones(3 * sc.n_pixels, dtype=torch.float32, device="cuda")
+        st = c.render_iteration(img, seed=4, iteration=0, mode=mars.MARS_MODE_WARMUP, profile=profile)
+        assert (img == 0).all() and st["rays"] == st["vertices"] == sc.n_pixels
+        assert st["trace_work"] == [[2 * sc.n_pixels, 0, 0, 0], [0, 0, 0, 0]]
