@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(MAX_LIGHT_THREADS, MINB) k_light_path(const De
                                                                const int d, const int d1) {
   const IterArgs it = *itp;
   DevCounters* ctr = c.ctr;
-  if (ctr->overflow) return;  // the tile is re-rendered
+  if (overflowed(ctr)) return;  // the tile is re-rendered
   const unsigned long long lb = ctr->lbase[d], lc = light_samples(ctr, d, d1);
   const unsigned long long n = lb >= a.lcap ? 0ull : (lc < a.lcap - lb ? lc : a.lcap - lb);
   const unsigned long long vb = vertex_base(ctr, d);
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(MAX_LIGHT_THREADS, MINB) k_light_connect(const
                                                                   const int d) {
   const IterArgs it = *itp;
   DevCounters* ctr = c.ctr;
-  if (ctr->overflow) return;  // the tile is re-rendered
+  if (overflowed(ctr)) return;  // the tile is re-rendered
   const unsigned long long lb = ctr->lbase[d];
   const unsigned long long vb = vertex_base(ctr, d), vc = ctr->vcount[d];
   const unsigned long long n = vb >= a.vcap ? 0ull : (vc < a.vcap - vb ? vc : a.vcap - vb);

@@ -91,6 +91,13 @@ __device__ __forceinline__ f3 normalize(f3 a) { return a * (1.0f / sqrtf(dot(a, 
 __device__ __forceinline__ float lum(f3 c) { return sum3(0.2126f, c.x, 0.7152f, c.y, 0.0722f, c.z); }
 __device__ __forceinline__ bool nonzero(f3 c) { return c.x > 0.f || c.y > 0.f || c.z > 0.f; }
 
+// Whether the tile has overflowed, the same for every lane of a warp: a kernel of
+// another stream may raise the flag while the warp reads it, and a warp that took
+// both answers would enter its collective steps in part.
+__device__ __forceinline__ bool overflowed(const DevCounters* ctr) {
+  return __any_sync(0xffffffffu, ctr->overflow != 0u);
+}
+
 // ------------------------------------------------------------ intersection
 __device__ __forceinline__ bool hit_quad(const float4* q, f3 o, f3 d, float tmax, float& t_out) {
   const f3 p0 = xyz(q[0]), e1 = xyz(q[1]), e2 = xyz(q[2]);

@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(MAX_WAVE_THREADS, MINB) k_trace(const DevScene
   DevCounters* ctr = c.ctr;
   // after an overflow some slots of this wave were never written: stop, the
   // tile is re-rendered in smaller pieces
-  if (ctr->overflow) return;
+  if (overflowed(ctr)) return;
   extern __shared__ RayStage ray_stage[];
   const Wave w = wave_of(ctr, a, d);
   TraceWork tw;
@@ -212,7 +212,7 @@ template <int MINB>
 __global__ void __launch_bounds__(MAX_WAVE_THREADS, MINB) k_shadow(const DevScene s, const DevCache c, const Arena a,
                                                            const int d, const int d1) {
   DevCounters* ctr = c.ctr;
-  if (ctr->overflow) return;
+  if (overflowed(ctr)) return;
   extern __shared__ RayStage ray_stage[];
   TraceWork tw;
   for (int e = d; e <= d1; ++e) {
