@@ -1164,6 +1164,7 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
     // were allocated; with the remaining waves taken as large as those, it
     // needed about demand x D / dstar slots (at least a halving, at most 16).
     int k = 2;
+    bool arena_full = false;  // more rays were drawn than the arena holds
     {
       const DevCounters& hc = *c->h_ctr;
       int dstar = 1;
@@ -1172,24 +1173,28 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
       const double est = (double)hc.demand * (double)D / (double)dstar;
       const double tcap = (double)(c->arena.cap / (uint64_t)std::max(1, nl));
       k = std::min(16, std::max(2, (int)std::ceil(1.3 * est / tcap)));
+      arena_full = (double)hc.demand > tcap;
     }
     std::vector<std::pair<int64_t, int64_t>> again;
+    bool slice_overflow = false;
     for (size_t t = 0; t < tiles.size(); ++t) {
       if (!c->h_tile_status[t]) continue;
       const int64_t a = tiles[t].first, b = tiles[t].second;
-      if (b - a <= 1 && !(tail > 0 && !(c->techniques & MARS_TECH_LIGHT)))
+      // a tile that only k_tail's slices were too small for goes to the wave kernels
+      // whole, which have all of the arena for it
+      const bool slices = c->h_tile_status[t] == OVER_SLICE && !arena_full;
+      if (b - a <= 1 && !slices)
         return set_error(MARS_ERR_OOM, "one pixel's path tree needs more than the arena's %llu rays",
                          (unsigned long long)(c->arena.cap / (uint64_t)std::max(1, nl)));
-      // a tile that k_tail's slices were too small for goes to the wave kernels whole,
-      // which have all of the arena for it
-      const int64_t parts = tail > 0 && !(c->techniques & MARS_TECH_LIGHT) ? 1 : std::min<int64_t>(k, b - a);
+      const int64_t parts = slices ? 1 : std::min<int64_t>(k, b - a);
+      slice_overflow = slice_overflow || c->h_tile_status[t] == OVER_SLICE;
       for (int64_t j = 0; j < parts; ++j) again.emplace_back(a + (b - a) * j / parts, a + (b - a) * (j + 1) / parts);
     }
     if (again.empty()) break;
     if ((int)again.size() > c->max_tiles) return set_error(MARS_ERR_OOM, "too many tiles after arena overflow");
     retries += (uint32_t)again.size();
     tiles.swap(again);
-    if (tail > 0) c->tail_margin = std::min(64.0, 2.0 * c->tail_margin);
+    if (slice_overflow) c->tail_margin = std::min(64.0, 2.0 * c->tail_margin);
     tail = 0;  // the wave kernels render them
     // the committed tiles stay; clear the overflow marker so the image pass runs
     if ((e = cudaMemsetAsync(&c->d_ctr->any_overflow, 0, sizeof(unsigned int), st)) != cudaSuccess)

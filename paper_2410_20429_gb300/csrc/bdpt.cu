@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(MAX_LIGHT_THREADS, MINB) k_light_path(const De
     const unsigned long long vfirst = vb + wb + (unsigned long long)(sc.x - m);
     if (active) {
       if (m > 0 && vfirst + (unsigned long long)m > a.vcap) {
-        atomicOr(&ctr->overflow, 1u);
+        atomicOr(&ctr->overflow, OVER_ARENA);
         m = 0;
       }
       // what the connections' weights need of each light vertex: its cell, the

@@ -147,6 +147,9 @@ constexpr uint32_t F_EST = 1u << 25;
 // of the grid serialise
 constexpr int IMG_SLOTS = 32;
 
+// a tile's overflow: of the arena by its waves, or of a block's slice in k_tail
+constexpr unsigned OVER_ARENA = 1u, OVER_SLICE = 2u;
+
 // rounds a block of k_tail may take
 constexpr int TAIL_ROUNDS = 96;
 
@@ -222,7 +225,7 @@ struct DevCache {
   float4* run_sum;      // [pixels]
   float4* img;          // [pixels] this iteration's image
   DevCounters* ctr;
-  unsigned int* tile_status;  // [max tiles] overflow per tile of the current attempt
+  unsigned int* tile_status;  // [max tiles] OVER_ bits per tile of the current attempt
   uint4* tail_rounds;         // k_tail's rounds: [blocks][TAIL_ROUNDS] (first child, rays, children, first root),
                               // then [blocks] (rounds, -, -, -); one such buffer per lane
   // adaptive octree over the scene box (oct_nodes null: the uniform grid).

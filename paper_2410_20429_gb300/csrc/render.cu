@@ -166,7 +166,7 @@ struct GridWave {
     b[2] = tl > 0 ? atomicAdd(&ctr->lcount[d], (Index)tl) : 0;
   }
   __device__ __forceinline__ Index list(int n_) { return atomicAdd(&ctr->slcount[d], (Index)n_); }
-  __device__ __forceinline__ void overflow() { atomicOr(&ctr->overflow, 1u); }
+  __device__ __forceinline__ void overflow() { atomicOr(&ctr->overflow, OVER_ARENA); }
 };
 
 template <int MINB, bool BD>

@@ -72,7 +72,7 @@ struct BlockWave {
     b[2] = 0;
   }
   __device__ __forceinline__ Index list(int n_) { return atomicAdd(slcount, (unsigned)n_); }
-  __device__ __forceinline__ void overflow() { *over = 1u; }
+  __device__ __forceinline__ void overflow() { *over = OVER_SLICE; }
 };
 constexpr int TAIL_THREADS = 128;
 constexpr int TAIL_WARPS = TAIL_THREADS / 32;
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(TAIL_THREADS, TAIL_BLOCKS) k_tail(const DevSce
   __syncthreads();
   if (tid == 0) {
     c.tail_rounds[(size_t)gridDim.x * TAIL_ROUNDS + blockIdx.x] = make_uint4((unsigned)r, 0u, 0u, 0u);
-    if (sh.over) atomicOr(&ctr->overflow, 1u);
+    if (sh.over & OVER_SLICE) atomicOr(&ctr->overflow, OVER_SLICE);
     if (sh.shadow_entries) atomicAdd(&ctr->scount[k], sh.shadow_entries);
     if (sh.shadow_traced) atomicAdd(&ctr->slcount[k], sh.shadow_traced);
   }

@@ -138,3 +138,42 @@ def test_arena_demand_counts_every_depth(mars, w, h, D):
     a, b = _pair(mars, w, h, D, TECH3, 0.1, 0.6, lanes=1)
     assert a[1]["wave_launches"] > b[1]["wave_launches"]
     assert b[1]["arena_demand"] == a[1]["arena_demand"] == a[1]["wave_entries"]
+
+
+def _box_job(mars, w, h, cap, lo, hi, est, lanes=1):
+    """A MARS job of the box from given counts and a uniform pixel estimate: (cache, next iteration)."""
+    import torch
+    cfg = W.config_box(w, h)
+    stream = torch.cuda.Stream()
+    scene = mars.Scene(cfg.scene, stream=stream)
+    c = mars.Cache(scene, cfg.grid_n, cfg.techniques, cfg.max_depth, arena_capacity=cap, lanes=lanes, stream=stream)
+    q_rr, q_s, valid = W.random_count_fields(cfg.n_cells, seed=41, lo=lo, hi=hi)
+    img = torch.zeros(3 * cfg.scene.n_pixels, dtype=torch.float32, device="cuda")
+    c.set_state(q_rr=q_rr, q_s=q_s, valid=valid, pixel_estimate=np.full((cfg.scene.n_pixels, 3), est, np.float32),
+                has_estimate=True, n_iterations=1, stream=stream)
+
+    def step(it, **kw):
+        kw = {"mode": mars.MARS_MODE_MARS, "update_estimate": False, **kw}
+        r = c.render_iteration(img, seed=3, iteration=it, stream=stream, **kw)
+        torch.cuda.synchronize()
+        return r, img.cpu().numpy().copy()
+
+    def estimate(e):
+        c.set_state(pixel_estimate=e, has_estimate=True, n_iterations=1, stream=stream)
+    return c, step, estimate
+
+
+@pytest.mark.parametrize("cap", [400000, 280000])
+def test_a_tile_the_arena_does_not_hold_is_split_at_once(mars, cap):
+    """Counts that jump: the rays fill the arena, in k_tail or in a wave before it.
+    The tile is split, without a second attempt as it is, into no more pieces than
+    after the wave kernels' own attempt (whose estimate of the rays it lacks differs)."""
+    out = []
+    for profile in (True, False):
+        c, step, estimate = _box_job(mars, 300, 260, cap, 0.05, 0.1, 0.5)
+        step(1, profile=profile)
+        estimate(np.full((c.n_pixels, 3), 0.01, np.float32))
+        out.append(step(2, profile=profile))
+    (a, ia), (b, ib) = out
+    assert 1 < b["retries"] <= a["retries"] and b["tiles"] <= a["tiles"]
+    assert np.array_equal(ia, ib) and a["rays"] == b["rays"]
