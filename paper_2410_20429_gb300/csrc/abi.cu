@@ -840,25 +840,32 @@ static DevCache lane_cache(const mars_cache* c, int l) {
 // iteration's rays per pixel (the first wave's is known), if what the waves
 // before leave of the arena holds the rest with tail_margin to spare -- a block's
 // subtrees may be larger than the average -- and, from the first wave on, 1.5 rays
-// per pixel and depth (a job's first iterations have little or no history).
+// per pixel and depth (a job's first iterations have little or no history).  The
+// NEE samples must fit as well, taken as spread over the waves like their rays.
+// tail_margin doubles when slices overflow and comes back down by half in 64
+// iterations without one, so that a job whose subtrees stay uneven pays for a
+// failed attempt once in that many and one whose counts settle gets its tail back.
 // kTailRays: at 30 000, 60 000, 120 000 and 250 000 the 512^2 room's warm-up took
 // 0.833, 0.819, 0.821 and 0.875 ms, its iterations with learned counts 1.159, 1.153,
 // 1.177 and 1.340, the heightfield at 1024^2 2.44, 2.40, 2.46 and 2.51; without
 // k_tail 0.844, 1.165 and 2.63.  Larger waves fill the GPU by themselves.
 constexpr double kTailRays = 65536.0;
+constexpr double kTailMargin = 2.0, kTailMarginMost = 1 << 20;
 static int tail_depth(const mars_cache* c, int64_t pixels, uint64_t cap) {
   const bool light = (c->techniques & MARS_TECH_LIGHT) != 0;
   if (!light && (c->tail_blocks <= 0 || cap > (1ull << 31))) return 0;
   const double scale = c->last_pixels > 0 ? (double)pixels / (double)c->last_pixels : 0.0;
   double before = 0.0, after = 0.0;
   for (int d = 1; d <= c->max_depth; ++d) after += scale * (double)c->last_wave[d];
+  const double shadow = after > 0.0 ? scale * (double)c->last_shadow / after : 0.0;  // NEE samples a ray
   for (int k = 1; k <= c->max_depth; ++k) {
     if (k > 1 && c->last_pixels == 0) return 0;
     const double wave = k == 1 ? (double)pixels : scale * (double)c->last_wave[k];
+    const bool shadow_fits = (double)cap - shadow * before >= c->tail_margin * shadow * after;
     before += wave;
     after -= scale * (double)c->last_wave[k];
     const double least = k == 1 ? 1.5 * (c->max_depth - 1) * (double)pixels : 0.0;
-    if (wave <= kTailRays && (light || (double)cap - before >= std::max(c->tail_margin * after, least))) return k;
+    if (wave <= kTailRays && (light || (shadow_fits && (double)cap - before >= std::max(c->tail_margin * after, least)))) return k;
   }
   return 0;
 }
@@ -976,6 +983,7 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
   // the first attempt of an iteration that needs one tile per lane may end in
   // k_tail (a profiled one times the wave kernels)
   int tail = 0;
+  bool slices_held = true;
   if (!p->profile && ntiles == iter_lanes) tail = tail_depth(c, nr / iter_lanes, c->arena.cap / (uint64_t)iter_lanes);
   uint64_t demand = 0;
   double trace_ms = 0.0, shade_ms = 0.0, shadow_ms = 0.0, reverse_ms = 0.0, image_ms = 0.0, light_ms = 0.0;
@@ -1194,7 +1202,10 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
     if ((int)again.size() > c->max_tiles) return set_error(MARS_ERR_OOM, "too many tiles after arena overflow");
     retries += (uint32_t)again.size();
     tiles.swap(again);
-    if (slice_overflow) c->tail_margin = std::min(64.0, 2.0 * c->tail_margin);
+    if (slice_overflow) {
+      c->tail_margin = std::min(kTailMarginMost, 2.0 * c->tail_margin);
+      slices_held = false;
+    }
     tail = 0;  // the wave kernels render them
     // the committed tiles stay; clear the overflow marker so the image pass runs
     if ((e = cudaMemsetAsync(&c->d_ctr->any_overflow, 0, sizeof(unsigned int), st)) != cudaSuccess)
@@ -1219,7 +1230,9 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
     c->next_tiles = std::min(c->max_tiles, std::max(1, t));
     c->last_entries = h.entries;
     for (int d = 1; d <= D; ++d) c->last_wave[d] = h.wave_total[d];
+    c->last_shadow = h.shadow_entries;
     c->last_pixels = nr;
+    if (slices_held) c->tail_margin = std::max(kTailMargin, c->tail_margin * 0.98922801319397548);  // 2^(-1/64)
     c->last_need = need;
   }
   if (p->update_estimate) {

@@ -38,6 +38,10 @@ struct Roots {
   __device__ __forceinline__ unsigned at(unsigned j) const {  // the wave's ray that is the block's root j
     return (j / ROOT_GROUP * blocks + block) * ROOT_GROUP + j % ROOT_GROUP;
   }
+  // blocks of `blocks` that have roots in a wave of n rays: the first ones
+  __device__ __forceinline__ static unsigned sharers(unsigned n, unsigned blocks) {
+    return max(1u, min(blocks, (n + ROOT_GROUP - 1) / ROOT_GROUP));
+  }
   __device__ __forceinline__ unsigned count(unsigned n) const {  // of a wave of n rays
     const unsigned groups = (n + ROOT_GROUP - 1) / ROOT_GROUP;
     if (block >= groups) return 0;
@@ -128,10 +132,13 @@ __global__ void __launch_bounds__(TAIL_THREADS, TAIL_BLOCKS) k_tail(const DevSce
   if (tid < 2) sh.count[tid] = sh.scount[tid] = sh.slcount[tid] = sh.next[0][tid] = sh.next[1][tid] = 0;
   __syncthreads();
   const IterArgs& it = sh.it;
-  // the block's slices of what the waves up to k left of the two regions
+  // the block's slices of what the waves up to k left of the two regions, shared by
+  // the blocks that have roots
+  const unsigned sharers = Roots::sharers((unsigned)w.n, gridDim.x);
   const unsigned long long start = w.base + w.n, sstart = k == 1 ? 0ull : ctr->sbase[k - 1] + ctr->scount[k - 1];
-  const unsigned slice = (unsigned)((a.cap - start) / gridDim.x);
-  const unsigned sslice = sstart < a.scap ? (unsigned)((a.scap - sstart) / gridDim.x) : 0u;
+  const bool sharer = blockIdx.x < sharers;
+  const unsigned slice = sharer ? (unsigned)((a.cap - start) / sharers) : 0u;
+  const unsigned sslice = sharer && sstart < a.scap ? (unsigned)((a.scap - sstart) / sharers) : 0u;
   RoundSlots rs;
   rs.base = (unsigned)start + blockIdx.x * slice;
   rs.n_child = rs.j0 = 0;

@@ -177,3 +177,37 @@ def test_a_tile_the_arena_does_not_hold_is_split_at_once(mars, cap):
     (a, ia), (b, ib) = out
     assert 1 < b["retries"] <= a["retries"] and b["tiles"] <= a["tiles"]
     assert np.array_equal(ia, ib) and a["rays"] == b["rays"]
+
+
+def test_the_tail_comes_back_after_its_slices_overflowed(mars):
+    """Three iterations whose few dear pixels overflow their blocks' slices, then even
+    ones: k_tail renders whole path trees again."""
+    c, step, estimate = _box_job(mars, 64, 64, 40000, 0.2, 0.5, 0.5)
+    even = np.full((c.n_pixels, 3), 0.5, np.float32)
+    dear = even.copy()
+    dear[2000:2004] = 2e-3
+    log = []
+    for it in range(1, 160):
+        if it <= 4:
+            estimate(dear if it < 4 else even)
+        log.append(step(it)[0])
+    assert log[0]["retries"] > 0 and all(r["retries"] == 0 for r in log[4:])
+    assert log[4]["wave_launches"] > 0 and log[-1]["wave_launches"] == 0
+
+
+def test_nee_samples_that_overflow_their_slices_are_learned(mars):
+    """Many more NEE samples than rays: one iteration finds out that the slices of the
+    shadow region are too small, the next ones know."""
+    import torch
+    cfg = W.config_box(64, 64)
+    stream = torch.cuda.Stream()
+    scene = mars.Scene(cfg.scene, stream=stream)
+    c = mars.Cache(scene, cfg.grid_n, cfg.techniques, cfg.max_depth, arena_capacity=30000, stream=stream)
+    q = np.zeros((c.n_cells, 3, 3), np.float32)
+    q[:, 0], q[:, 1] = 0.02, 1.0
+    c.set_state(q_rr=q, q_s=0.9 * q, valid=np.ones((c.n_cells, 3), np.uint8), has_estimate=True, n_iterations=1,
+                pixel_estimate=np.full((c.n_pixels, 3), 0.5, np.float32), stream=stream)
+    log = [c.render_iteration(None, seed=2, iteration=it, mode=mars.MARS_MODE_MARS, update_estimate=False,
+                              stream=stream) for it in range(1, 8)]
+    assert log[0]["shadow_entries"] > 2 * log[0]["wave_entries"]
+    assert all(r["retries"] == 0 for r in log[1:])
