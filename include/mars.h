@@ -130,8 +130,11 @@ typedef struct {
  *   default an iteration whose pixel tiles fit the arena at the first attempt,
  *   is not profiled and runs on a stream other than the legacy default stream
  *   (which cannot be captured) is recorded once as a CUDA graph and replayed;
- *   the graph is recorded again when the output buffer, update_estimate, the
- *   image-statistics options, the tile count or the launch shape change.
+ *   another graph is recorded when the output buffer, update_estimate, the
+ *   image-statistics options, the pixel range, the tile count, the launch shape or
+ *   the depth from which on the small waves are rendered together change.  The
+ *   last four are kept.  The first iteration of an image of more than 2^16 pixels,
+ *   which has yet to tell that depth, launches its kernels directly.
  *   MARS_CACHE_ONE_LANE: one tile lane.  By default the pixels are split into
  *   tiles dealt to two lanes, each with half the arena, its own streams and
  *   counters, rendered concurrently (their wave kernels fill each other's idle

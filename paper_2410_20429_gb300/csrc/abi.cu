@@ -805,7 +805,7 @@ void cache_destroy_impl(mars_cache* c) {
   dev_free(c->d_args, st);
   dev_free(c->d_host_stage, st);
   pinned_release(c->h_args, sizeof(IterArgs) * c->max_tiles);
-  if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
+  for (auto& g : c->graphs) cudaGraphExecDestroy(g.exec);
   for (cudaEvent_t ev : c->events) cudaEventDestroy(ev);
   for (cudaEvent_t ev : c->sync_events) cudaEventDestroy(ev);
   for (auto& v : c->lane_sync)
@@ -850,6 +850,10 @@ static DevCache lane_cache(const mars_cache* c, int l) {
 // 1.177 and 1.340, the heightfield at 1024^2 2.44, 2.40, 2.46 and 2.51; without
 // k_tail 0.844, 1.165 and 2.63.  Larger waves fill the GPU by themselves.
 constexpr double kTailRays = 65536.0;
+// A depth in use is kept while its wave stays below kTailBand times that and no
+// earlier wave falls as far below it: next to the best depth the time changes by 1
+// or 2 %, and another depth is another recording of the iteration's graph.
+constexpr double kTailBand = 1.5;
 constexpr double kTailMargin = 2.0, kTailMarginMost = 1 << 20;
 static int tail_depth(const mars_cache* c, int64_t pixels, uint64_t cap) {
   const bool light = (c->techniques & MARS_TECH_LIGHT) != 0;
@@ -858,16 +862,22 @@ static int tail_depth(const mars_cache* c, int64_t pixels, uint64_t cap) {
   double before = 0.0, after = 0.0;
   for (int d = 1; d <= c->max_depth; ++d) after += scale * (double)c->last_wave[d];
   const double shadow = after > 0.0 ? scale * (double)c->last_shadow / after : 0.0;  // NEE samples a ray
-  for (int k = 1; k <= c->max_depth; ++k) {
-    if (k > 1 && c->last_pixels == 0) return 0;
+  int rule = 0;       // the rule's depth
+  double at = 0.0;    // and its wave
+  bool stay = false;  // the last iteration's depth still serves
+  for (int k = 1; k <= c->max_depth && (k == 1 || c->last_pixels > 0); ++k) {
     const double wave = k == 1 ? (double)pixels : scale * (double)c->last_wave[k];
     const bool shadow_fits = (double)cap - shadow * before >= c->tail_margin * shadow * after;
     before += wave;
     after -= scale * (double)c->last_wave[k];
     const double least = k == 1 ? 1.5 * (c->max_depth - 1) * (double)pixels : 0.0;
-    if (wave <= kTailRays && (light || (shadow_fits && (double)cap - before >= std::max(c->tail_margin * after, least)))) return k;
+    if (!light && !(shadow_fits && (double)cap - before >= std::max(c->tail_margin * after, least))) continue;
+    if (rule == 0 && wave <= kTailRays) rule = k, at = wave;
+    if (k > 1 && k == c->last_tail && wave <= kTailBand * kTailRays) stay = true;
   }
-  return 0;
+  if (stay && rule != c->last_tail && (rule == 0 || rule > c->last_tail || kTailBand * at > kTailRays))
+    return c->last_tail;
+  return rule;
 }
 
 // lane l's share of the arena when nl lanes are in use: the l-th of nl equal
@@ -982,9 +992,11 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
   uint32_t retries = 0, used = 0, launches = 0, wave_launches = 0;
   // the first attempt of an iteration that needs one tile per lane may end in
   // k_tail (a profiled one times the wave kernels)
+  const bool first = c->last_pixels == 0 && nr / iter_lanes > (int64_t)kTailRays;
   int tail = 0;
   bool slices_held = true;
   if (!p->profile && ntiles == iter_lanes) tail = tail_depth(c, nr / iter_lanes, c->arena.cap / (uint64_t)iter_lanes);
+  const int first_tail = p->profile ? c->last_tail : tail;
   uint64_t demand = 0;
   double trace_ms = 0.0, shade_ms = 0.0, shadow_ms = 0.0, reverse_ms = 0.0, image_ms = 0.0, light_ms = 0.0;
   float wave_ms[WAVE_KERNELS][MAXD] = {};
@@ -1085,9 +1097,11 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
     // A first attempt with at most one tile per lane is replayed from a
     // recorded CUDA graph.  The legacy default stream cannot be captured, and a
     // profiled iteration times every launch with stream events: both launch
-    // directly, as do the re-rendered tiles after an arena overflow.
+    // directly, as do the re-rendered tiles after an arena overflow and a job's
+    // first iteration where its waves have yet to tell the tail's depth (its graph
+    // would be of use once).
     const bool capturable = st != nullptr && st != cudaStreamLegacy && st != cudaStreamPerThread;
-    if (c->use_graphs && capturable && !profile && retries == 0 && (int)tiles.size() <= iter_lanes) {
+    if (c->use_graphs && capturable && !profile && retries == 0 && (int)tiles.size() <= iter_lanes && !first) {
       GraphKey key;
       key.tiles = (int)tiles.size();
       key.tail = tail;
@@ -1098,11 +1112,16 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
       key.r0 = ranged ? r0 : 0;
       key.r1 = ranged ? r1 : 0;
       key.L = c->launch;
-      if (!c->graph_exec || !(c->graph_key == key)) {
-        if (c->graph_exec) {
-          cudaGraphExecDestroy(c->graph_exec);
-          c->graph_exec = nullptr;
-        }
+      // The last few are kept: a job that goes back and forth between tail depths,
+      // modes or image buffers records each once.  The iteration that finds none is
+      // launched directly, and its graph recorded while the GPU works on it: a
+      // recording takes the host about a quarter of a 512^2 iteration's time.
+      auto found = std::find_if(c->graphs.begin(), c->graphs.end(), [&](const auto& g) { return g.key == key; });
+      if (found != c->graphs.end()) {
+        std::rotate(c->graphs.begin(), found, found + 1);
+        if ((e = cudaGraphLaunch(c->graphs.front().exec, st)) != cudaSuccess) return poison(c, e, "graph launch");
+      } else {
+        if ((e = enqueue(st)) != cudaSuccess) return poison(c, e, "render launch");
         NvtxRange nvtx_capture("mars:graph_capture");
         cudaGraph_t graph = nullptr;
         if ((e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
@@ -1113,16 +1132,17 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
           if (graph) cudaGraphDestroy(graph);
           return poison(c, ee != cudaSuccess ? ee : e, "graph capture");
         }
-        e = cudaGraphInstantiate(&c->graph_exec, graph, 0);
+        cudaGraphExec_t exec = nullptr;
+        e = cudaGraphInstantiate(&exec, graph, 0);
         cudaGraphDestroy(graph);
-        if (e != cudaSuccess) {
-          c->graph_exec = nullptr;
-          return poison(c, e, "graph instantiate");
+        if (e != cudaSuccess) return poison(c, e, "graph instantiate");
+        if (c->graphs.size() == mars_cache::kMaxGraphs) {
+          cudaGraphExecDestroy(c->graphs.back().exec);
+          c->graphs.pop_back();
         }
-        c->graph_key = key;
+        c->graphs.insert(c->graphs.begin(), {key, exec});
         c->graph_captures += 1;
       }
-      if ((e = cudaGraphLaunch(c->graph_exec, st)) != cudaSuccess) return poison(c, e, "graph launch");
     } else if ((e = enqueue(st)) != cudaSuccess) {
       return poison(c, e, "render launch");
     }
@@ -1230,6 +1250,7 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
     c->next_tiles = std::min(c->max_tiles, std::max(1, t));
     c->last_entries = h.entries;
     for (int d = 1; d <= D; ++d) c->last_wave[d] = h.wave_total[d];
+    c->last_tail = first_tail;
     c->last_shadow = h.shadow_entries;
     c->last_pixels = nr;
     if (slices_held) c->tail_margin = std::max(kTailMargin, c->tail_margin * 0.98922801319397548);  // 2^(-1/64)

@@ -132,6 +132,7 @@ struct mars_cache {
   uint64_t last_shadow = 0;        // NEE samples of the last iteration
   uint64_t last_wave[mars::MAXD + 2] = {};  // rays per depth of the last iteration
   int64_t last_pixels = 0;                  // and its pixels
+  int last_tail = 0;                        // the depth from which on it ran in k_tail
   int max_tiles = 0;
   int next_tiles = 1;
   int n_iterations = 0;
@@ -172,10 +173,14 @@ struct mars_cache {
   double* d_comb_w = nullptr;     // its weight sum
   double* d_img_acc = nullptr;    // V_I and C_I sums since the last update, and their count
   unsigned long long* d_topk = nullptr;  // brightest-pixel candidates
-  // the recorded single-tile iteration graph (MARS_CACHE_NO_GRAPHS: none)
+  // the recorded iteration graphs, the last used first (MARS_CACHE_NO_GRAPHS: none)
   bool use_graphs = true;
-  cudaGraphExec_t graph_exec = nullptr;
-  mars::GraphKey graph_key{};
+  struct Recorded {
+    mars::GraphKey key;
+    cudaGraphExec_t exec;
+  };
+  static constexpr size_t kMaxGraphs = 4;
+  std::vector<Recorded> graphs;
   int graph_captures = 0;
 };
 

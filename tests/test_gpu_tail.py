@@ -211,3 +211,38 @@ def test_nee_samples_that_overflow_their_slices_are_learned(mars):
                               stream=stream) for it in range(1, 8)]
     assert log[0]["shadow_entries"] > 2 * log[0]["wave_entries"]
     assert all(r["retries"] == 0 for r in log[1:])
+
+
+def test_a_steady_job_records_one_graph(mars):
+    """An image of more than 2^16 pixels: the first iteration tells the depth of the
+    tail, the next records the graph that all others replay."""
+    c, step, _ = _box_job(mars, 300, 260, 0, 0.1, 0.3, 0.5)
+    caps = []
+    for it in range(6):
+        step(it, mode=mars.MARS_MODE_WARMUP)
+        caps.append(c.info()["graph_captures"])
+    assert caps == [0, 1, 1, 1, 1, 1]
+
+
+@pytest.mark.parametrize("w,h", [(310, 270), (480, 360)])
+def test_a_job_that_alternates_records_each_graph_once(mars, w, h):
+    """Fixed counts and learned ones in turn, whose waves call for two depths of the
+    tail: the graph of each is recorded once."""
+    c, step, _ = _box_job(mars, w, h, 0, 0.1, 0.3, 0.5)
+    rays = [step(it, mode=(mars.MARS_MODE_FIXED, mars.MARS_MODE_MARS)[it & 1])[0]["wave_rays"][1] for it in range(12)]
+    assert min(rays[::2]) > 65536 > max(rays[1::2])
+    assert c.info()["graph_captures"] <= 2
+
+
+def test_graphs_kept_are_few_and_replay_their_own_settings(mars):
+    """Six settings in turn, more than are kept: each gives the image it gave at first."""
+    c, step, _ = _box_job(mars, 64, 48, 0, 0.1, 0.3, 0.5)
+    shapes = [([t] * 4, [0] * 4) for t in (32, 64, 96, 128, 160, 256)]
+    first = None
+    for it in range(3):
+        for s in shapes:
+            c.set_launch(*s)
+            r, img = step(7, collect=False)
+            first = img if first is None else first
+            assert np.array_equal(img, first)
+    assert c.info()["graph_captures"] == 18
