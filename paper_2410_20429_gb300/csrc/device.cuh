@@ -53,8 +53,9 @@ __device__ __forceinline__ f3 operator*(f3 a, float s) { return {a.x * s, a.y * 
 __device__ __forceinline__ f3 mul(f3 a, f3 b) { return {a.x * b.x, a.y * b.y, a.z * b.z}; }
 // Sums of products.  The compiler may fuse either product of a * b + c * d into
 // the addition, and which one it takes depends on the code around it.
-// MARS_PIN_FMA spells out the choice it makes in the wave kernels, for a
-// translation unit whose kernels have to give their results bit for bit.
+// MARS_PIN_FMA spells out the choice it makes in the unidirectional wave kernels,
+// for a translation unit whose kernels have to give their results bit for bit
+// (tests/test_gpu_tail.py compares them; the bidirectional kernels take others).
 #ifdef MARS_PIN_FMA
 __device__ __forceinline__ float sum2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
 __device__ __forceinline__ float diff2(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
@@ -70,16 +71,18 @@ __device__ __forceinline__ float sum3(float a, float b, float c, float d, float 
 #endif
 }
 __device__ __forceinline__ float dot(f3 a, f3 b) { return sum3(a.x, b.x, a.y, b.y, a.z, b.z); }
+// the first two products fused the other way round
+__device__ __forceinline__ float dot_yx(f3 a, f3 b) {
+#ifdef MARS_PIN_FMA
+  return __fmaf_rn(a.z, b.z, __fmaf_rn(a.y, b.y, __fmul_rn(a.x, b.x)));
+#else
+  return dot(a, b);
+#endif
+}
 __device__ __forceinline__ f3 cross(f3 a, f3 b) {
   return {diff2(a.y, b.z, a.z, b.y), diff2(a.z, b.x, a.x, b.z), diff2(a.x, b.y, a.y, b.x)};
 }
-__device__ __forceinline__ float length2_hit(f3 a) {
-#ifdef MARS_PIN_FMA
-  return __fmaf_rn(a.z, a.z, __fmaf_rn(a.y, a.y, __fmul_rn(a.x, a.x)));
-#else
-  return dot(a, a);
-#endif
-}
+__device__ __forceinline__ float length2_hit(f3 a) { return dot_yx(a, a); }
 // a u + b v (+ c w)
 __device__ __forceinline__ f3 span2(f3 a, float u, f3 b, float v) {
   return {sum2(a.x, u, b.x, v), sum2(a.y, u, b.y, v), sum2(a.z, u, b.z, v)};
@@ -139,11 +142,17 @@ __device__ __forceinline__ bool hit_tri(const float4* q, f3 o, f3 d, float tmax,
   if (det == 0.0f) return false;
   const float inv = 1.0f / det;
   const f3 s = o - v0;
-  const float a = dot(s, p) * inv;
+  const float sa = dot_yx(s, p);
+  const float a = sa * inv;
   if (a < 0.0f || a > 1.0f) return false;
   const f3 qv = cross(s, e1);
   const float b = dot(d, qv) * inv;
-  if (b < 0.0f || a + b > 1.0f) return false;
+#ifdef MARS_PIN_FMA
+  const float ab = __fmaf_rn(sa, inv, b);
+#else
+  const float ab = a + b;
+#endif
+  if (b < 0.0f || ab > 1.0f) return false;
   const float t = dot(e2, qv) * inv;
   if (!(t > 0.0f && t < tmax)) return false;
   t_out = t;

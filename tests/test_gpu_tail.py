@@ -246,3 +246,67 @@ def test_graphs_kept_are_few_and_replay_their_own_settings(mars):
             first = img if first is None else first
             assert np.array_equal(img, first)
     assert c.info()["graph_captures"] == 18
+
+
+def _both(mars, c, step):
+    """An iteration by the wave kernels and by k_tail: images, counters and rays of every pixel the same."""
+    out = []
+    for profile in (True, False):
+        r, img = step(profile)
+        out.append((img, r, c.get_state()["pixel_rays"]))
+    (ia, ra, pa), (ib, rb, pb) = out
+    assert rb["wave_launches"] == 0 and np.array_equal(ia, ib) and np.array_equal(pa, pb)
+    for k in KEYS:
+        assert ra[k] == rb[k], k
+
+
+FORMS = {"triangles": dict(tech=3), "guided_triangles": {}, "lbvh": {}, "many_spheres": {}, "warmup": dict(mode=0),
+         "octree": dict(grid=4, cache=dict(octree=True, max_leaves=4096, split_samples=40.0)),
+         "fixed": dict(mode=2), "unaware": dict(kw=dict(weights=1)), "fixed_unaware": dict(mode=2, kw=dict(weights=1)),
+         "float32": dict(cache=dict(fp32_statistics=True)), "capped": dict(kw=dict(max_multiplicity=4.0))}
+
+
+@pytest.mark.parametrize("form", FORMS)
+def test_every_form_of_an_iteration_equals_the_wave_kernels(mars, form):
+    import torch
+    f = FORMS[form]
+    tech = f.get("tech", TECH3)
+    sc = W.guided_room_scene(2, 97, 61, n_spheres=900 if form == "many_spheres" else 24)
+    if form in ("triangles", "guided_triangles", "lbvh"):
+        sc = W.heightfield_scene(3, 40, 97, 61, n_spheres=30, n_lights=2, ggx_fraction=0.5)
+        sc.bvh = int(form == "lbvh")
+    scene = mars.Scene(sc)
+    c = mars.Cache(scene, f.get("grid", 6), tech, 7, **f.get("cache", {}))
+    img = torch.zeros(3 * sc.n_pixels, dtype=torch.float32, device="cuda")
+    if form == "octree":
+        c.render_iteration(img, seed=6, iteration=0, mode=mars.MARS_MODE_WARMUP)
+        c.update_counts()
+    q_rr, q_s, valid = W.random_count_fields(c.n_cells, seed=31, lo=0.1, hi=0.6)
+    state = dict(q_rr=q_rr, q_s=q_s, valid=valid, has_estimate=True, n_iterations=1,
+                 pixel_estimate=W.random_pixel_estimate(sc.n_pixels, seed=32, lo=0.2, hi=0.5))
+    if tech & W.TECH_GUIDED:
+        state["guide_cdf"] = W.random_guide_cdf(c.n_cells, 33)
+
+    def step(profile):
+        c.set_state(**state)
+        r = c.render_iteration(img, seed=6, iteration=3, mode=f.get("mode", 1), profile=profile, **f.get("kw", {}))
+        torch.cuda.synchronize()
+        return r, img.cpu().numpy().copy()
+    _both(mars, c, step)
+
+
+def test_rays_at_the_edges_of_triangles_equal_the_wave_kernels(mars):
+    """2.6 million camera rays and their second bounce over 131k triangles: one in some
+    hundred thousand meets an edge to within the rounding of the edge functions, and
+    which of two triangles it hits, or neither, is the same in both."""
+    import torch
+    sc = W.heightfield_scene(7, 256, 256, 256, n_spheres=64)
+    scene = mars.Scene(sc)
+    c = mars.Cache(scene, 8, 3, 3)
+    img = torch.zeros(3 * sc.n_pixels, dtype=torch.float32, device="cuda")
+    for it in range(40):
+        def step(profile):
+            r = c.render_iteration(img, seed=11, iteration=it, mode=mars.MARS_MODE_WARMUP, profile=profile)
+            torch.cuda.synchronize()
+            return r, img.cpu().numpy().copy()
+        _both(mars, c, step)
