@@ -836,7 +836,7 @@ static DevCache lane_cache(const mars_cache* c, int l) {
 // The depth from which on an iteration of `pixels` pixels a lane, with a ray arena
 // of `cap` slots a lane, runs in k_tail (with light connections: joins its waves'
 // side kernels, which needs no room); 0: nowhere.  The first wave of at most
-// kTailRays rays, its size and those of the deeper waves taken from the last
+// kTailRays rays over the lanes, its size and those of the deeper waves taken from the last
 // iteration's rays per pixel (the first wave's is known), if what the waves
 // before leave of the arena holds the rest with tail_margin to spare -- a block's
 // subtrees may be larger than the average -- and, from the first wave on, 1.5 rays
@@ -848,14 +848,20 @@ static DevCache lane_cache(const mars_cache* c, int l) {
 // kTailRays: at 30 000, 60 000, 120 000 and 250 000 the 512^2 room's warm-up took
 // 0.833, 0.819, 0.821 and 0.875 ms, its iterations with learned counts 1.159, 1.153,
 // 1.177 and 1.340, the heightfield at 1024^2 2.44, 2.40, 2.46 and 2.51; without
-// k_tail 0.844, 1.165 and 2.63.  Larger waves fill the GPU by themselves.
+// k_tail 0.844, 1.165 and 2.63.  Larger waves fill the GPU by themselves, and the
+// waves of two lanes fill it together: with 65536 rays a lane, twice that in all,
+// the 512^2 room with counts learned over 20 iterations rendered 1610 to 1652
+// Mvertices/s in two lanes, with 32768 a lane 1715 to 1719 and without k_tail 1705 to
+// 1725 (in one lane all three 1616 to 1644); a drawn room's learned-count iteration
+// 1.35 -> 1.26 ms, the heightfield at 1024^2 2.27 -> 2.23.
 constexpr double kTailRays = 65536.0;
 // A depth in use is kept while its wave stays below kTailBand times that and no
 // earlier wave falls as far below it: next to the best depth the time changes by 1
 // or 2 %, and another depth is another recording of the iteration's graph.
 constexpr double kTailBand = 1.5;
 constexpr double kTailMargin = 2.0, kTailMarginMost = 1 << 20;
-static int tail_depth(const mars_cache* c, int64_t pixels, uint64_t cap) {
+static int tail_depth(const mars_cache* c, int64_t pixels, uint64_t cap, int lanes) {
+  const double most = kTailRays / lanes;
   const bool light = (c->techniques & MARS_TECH_LIGHT) != 0;
   if (!light && (c->tail_blocks <= 0 || cap > (1ull << 31))) return 0;
   const double scale = c->last_pixels > 0 ? (double)pixels / (double)c->last_pixels : 0.0;
@@ -872,10 +878,10 @@ static int tail_depth(const mars_cache* c, int64_t pixels, uint64_t cap) {
     after -= scale * (double)c->last_wave[k];
     const double least = k == 1 ? 1.5 * (c->max_depth - 1) * (double)pixels : 0.0;
     if (!light && !(shadow_fits && (double)cap - before >= std::max(c->tail_margin * after, least))) continue;
-    if (rule == 0 && wave <= kTailRays) rule = k, at = wave;
-    if (k > 1 && k == c->last_tail && wave <= kTailBand * kTailRays) stay = true;
+    if (rule == 0 && wave <= most) rule = k, at = wave;
+    if (k > 1 && k == c->last_tail && wave <= kTailBand * most) stay = true;
   }
-  if (stay && rule != c->last_tail && (rule == 0 || rule > c->last_tail || kTailBand * at > kTailRays))
+  if (stay && rule != c->last_tail && (rule == 0 || rule > c->last_tail || kTailBand * at > most))
     return c->last_tail;
   return rule;
 }
@@ -992,10 +998,10 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
   uint32_t retries = 0, used = 0, launches = 0, wave_launches = 0;
   // the first attempt of an iteration that needs one tile per lane may end in
   // k_tail (a profiled one times the wave kernels)
-  const bool first = c->last_pixels == 0 && nr / iter_lanes > (int64_t)kTailRays;
+  const bool first = c->last_pixels == 0 && nr > (int64_t)kTailRays;
   int tail = 0;
   bool slices_held = true;
-  if (!p->profile && ntiles == iter_lanes) tail = tail_depth(c, nr / iter_lanes, c->arena.cap / (uint64_t)iter_lanes);
+  if (!p->profile && ntiles == iter_lanes) tail = tail_depth(c, nr / iter_lanes, c->arena.cap / (uint64_t)iter_lanes, iter_lanes);
   const int first_tail = p->profile ? c->last_tail : tail;
   uint64_t demand = 0;
   double trace_ms = 0.0, shade_ms = 0.0, shadow_ms = 0.0, reverse_ms = 0.0, image_ms = 0.0, light_ms = 0.0;

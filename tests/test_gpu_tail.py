@@ -310,3 +310,18 @@ def test_rays_at_the_edges_of_triangles_equal_the_wave_kernels(mars):
             torch.cuda.synchronize()
             return r, img.cpu().numpy().copy()
         _both(mars, c, step)
+
+
+@pytest.mark.parametrize("lanes", [1, 2])
+@pytest.mark.parametrize("w", [440, 560, 700, 880])
+def test_the_tail_starts_at_the_first_small_wave_of_all_lanes(mars, w, lanes):
+    """The wave of at most 2^16 rays is counted over the lanes, whose waves run at the
+    same time.  The depth comes from the iteration before: waves of that many pixels
+    differ from it by less than 5 %."""
+    c, step, _ = _box_job(mars, w, 300, 0, 0.1, 0.3, 0.5, lanes=lanes)
+    for it in range(2):
+        r, _ = step(it, mode=mars.MARS_MODE_WARMUP)
+    assert r["tiles"] == lanes and r["retries"] == 0
+    waves, before = r["wave_rays"], r["wave_launches"] // r["tiles"]  # waves of the wave kernels
+    assert all(n > 0.95 * 65536 for n in waves[:before])
+    assert before == len(waves) or waves[before] < 1.05 * 65536
