@@ -1708,7 +1708,8 @@ mars_status mars_cache_autotune(mars_cache* c, const mars_iter_params* params, i
       mars_iter_stats st{};
       rc = render_iteration_impl(c, &p, nullptr, &st, (cudaStream_t)stream);
       if (rc != MARS_OK) return rc;
-      const double v[WAVE_KERNELS] = {st.trace_ms, st.shade_ms, st.shadow_ms, st.reverse_ms};
+      // the light connection kernels take the shadow kernel's shape
+      const double v[WAVE_KERNELS] = {st.trace_ms, st.shade_ms, st.shadow_ms + st.light_ms, st.reverse_ms};
       if (r > 0) tot += v[k];
     }
     *ms = tot / repeats;
@@ -1720,7 +1721,7 @@ mars_status mars_cache_autotune(mars_cache* c, const mars_iter_params* params, i
     int best_t = threads[k], best_b = bps[k], best_v = var[k];
     double best = 1e300;
     for (int v = 0; v < wave_variants(k); ++v) {
-      if (wave_variant_repeats(k, v)) continue;
+      if (wave_variant_repeats(k, v, c->techniques)) continue;
       for (int ti = 0; ti < 3; ++ti) {
         int occ[WAVE_KERNELS];
         int tt[WAVE_KERNELS] = {threads[0], threads[1], threads[2], threads[3]};

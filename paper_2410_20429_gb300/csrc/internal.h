@@ -299,7 +299,9 @@ cudaError_t wave_occupancy(const int threads[WAVE_KERNELS], const int variant[WA
                            int blocks_per_sm[WAVE_KERNELS]);
 int wave_variants(int kernel);                    // compiled register-cap variants of a wave kernel
 int wave_variant_registers(int kernel, int v);    // its register cap (0: the library's choice)
-bool wave_variant_repeats(int kernel, int v);     // the same code as variant 0
+// the same code as variant 0 (with light connections the shadow kernel's variant is
+// the light kernels' too, whose variants all differ)
+bool wave_variant_repeats(int kernel, int v, int techniques);
 bool wave_threads_ok(int threads);
 int tile_launches(int max_depth, int techniques, int tail);  // kernels launch_tile issues
 // the waves from depth k on (tail.cu): forward, and in reverse over the same grid

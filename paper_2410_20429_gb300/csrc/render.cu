@@ -268,7 +268,9 @@ TraceFn reverse_fn(int v, bool bd = false) {
 }  // namespace
 
 int wave_variants(int) { return 3; }
-bool wave_variant_repeats(int kernel, int v) { return v == 1 && kernel != WK_REVERSE; }
+bool wave_variant_repeats(int kernel, int v, int techniques) {
+  return v == 1 && kernel != WK_REVERSE && !(kernel == WK_SHADOW && (techniques & MARS_TECH_LIGHT));
+}
 int wave_variant_registers(int kernel, int v) {
   if (v == 0) return 0;
   if (kernel == WK_SHADE || kernel == WK_REVERSE) return v == 1 ? 80 : 64;
