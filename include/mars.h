@@ -417,7 +417,9 @@ mars_status mars_cache_set_state(mars_cache* cache, const mars_cache_state* stat
  * threads[k]: threads per block of kernel k (0 trace, 1 shade, 2 shadow,
  *   3 reverse), a multiple of 32 in 32..256.
  * blocks_per_sm[k]: 1..64, or 0 = as many blocks as fit on an SM at once
- *   (mars_cache_get_launch reports the resolved count).
+ *   (mars_cache_get_launch reports the resolved count).  The kernels that render
+ *   the small waves together have 128 threads a block and up to four blocks an SM,
+ *   no more threads than the kernel with most has by threads x blocks_per_sm.
  * max_registers[k]: selects a compiled variant of the kernel whose registers
  *   per thread are capped (more resident blocks, possibly some spilling).
  * lanes: concurrent tile lanes an iteration may use, 1 up to the count the

@@ -771,6 +771,12 @@ mars_status apply_launch(mars_cache* c, const int threads[WAVE_KERNELS], const i
     c->launch.grid[k] = c->scene->num_sms * b;
     c->blocks_per_sm[k] = b;
   }
+  // k_tail stands in for the wave kernels: it takes no more threads of an SM than
+  // the shape gives to the one of them that has most (by default and after tuning
+  // more than k_tail can use; a caller who limits the blocks leaves room on purpose)
+  int most = 0;
+  for (int k = 0; k < WAVE_KERNELS; ++k) most = std::max(most, c->launch.threads[k] * c->blocks_per_sm[k]);
+  c->tail_grid = std::min(c->tail_blocks, c->scene->num_sms * std::max(1, most / TAIL_THREADS));
   return MARS_OK;
 }
 
@@ -1070,7 +1076,7 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
         const bool own = concurrent && l >= 1;
         cudaStream_t side2 = own ? (c->lane_side2.empty() ? nullptr : c->lane_side2[l - 1]) : c->side2;
         if ((r = launch_tile(s->ds, lane_cache(c, l), lane_arena(c, l, nl), c->d_args + t, c->launch,
-                             tiles[t].second - tiles[t].first, tail, std::max(1, c->tail_blocks / nl), own ? c->lane_st[l - 1] : q, own ? c->lane_side[l - 1] : c->side, side2,
+                             tiles[t].second - tiles[t].first, tail, std::max(1, c->tail_grid / nl), own ? c->lane_st[l - 1] : q, own ? c->lane_side[l - 1] : c->side, side2,
                              own ? c->lane_sync[l - 1].data() : c->sync_events.data(), ev)) != cudaSuccess)
           return r;
       }

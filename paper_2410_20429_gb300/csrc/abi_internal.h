@@ -128,6 +128,7 @@ struct mars_cache {
   unsigned int* h_tile_status = nullptr;
   uint4* d_tail_rounds = nullptr;  // one buffer per lane (see DevCache)
   int tail_blocks = 0;             // resident blocks of k_tail (0: it is not used)
+  int tail_grid = 0;               // those that the launch shape allows
   double tail_margin = 2.0;        // headroom of k_tail's slices over the last iteration's use
   uint64_t last_shadow = 0;        // NEE samples of the last iteration
   uint64_t last_wave[mars::MAXD + 2] = {};  // rays per depth of the last iteration

@@ -150,7 +150,8 @@ constexpr int IMG_SLOTS = 32;
 // a tile's overflow: of the arena by its waves, or of a block's slice in k_tail
 constexpr unsigned OVER_ARENA = 1u, OVER_SLICE = 2u;
 
-// rounds a block of k_tail may take
+// threads of a block of k_tail, rounds it may take
+constexpr int TAIL_THREADS = 128;
 constexpr int TAIL_ROUNDS = 96;
 
 // Device-resident per-iteration counters.

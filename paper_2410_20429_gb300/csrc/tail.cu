@@ -78,7 +78,6 @@ struct BlockWave {
   __device__ __forceinline__ Index list(int n_) { return atomicAdd(slcount, (unsigned)n_); }
   __device__ __forceinline__ void overflow() { *over = OVER_SLICE; }
 };
-constexpr int TAIL_THREADS = 128;
 constexpr int TAIL_WARPS = TAIL_THREADS / 32;
 // four blocks an SM: 126 registers and no spills (five blocks at 96 registers:
 // 128^2 room 0.48 -> 0.52 ms; the chain of one thread's instructions is what

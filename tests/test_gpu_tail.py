@@ -325,3 +325,22 @@ def test_the_tail_starts_at_the_first_small_wave_of_all_lanes(mars, w, lanes):
     waves, before = r["wave_rays"], r["wave_launches"] // r["tiles"]  # waves of the wave kernels
     assert all(n > 0.95 * 65536 for n in waves[:before])
     assert before == len(waves) or waves[before] < 1.05 * 65536
+
+
+@pytest.mark.parametrize("cap,threads,blocks", [(80000, 32, 1), (120000, 128, 2), (120000, 64, 4)])
+def test_k_tail_keeps_to_the_room_a_launch_shape_leaves(mars, cap, threads, blocks):
+    """Fewer blocks an SM than fit: k_tail has no more threads there than the wave
+    kernels, seen by its slices, which are the larger the fewer blocks share the
+    arena and then hold the subtrees of a few dear pixels."""
+    out = []
+    for shape in (None, ([threads] * 4, [blocks] * 4)):
+        c, step, estimate = _box_job(mars, 64, 64, cap, 0.2, 0.5, 0.5)
+        dear = np.full((c.n_pixels, 3), 0.5, np.float32)
+        dear[2000:2004] = 2e-3
+        estimate(dear)
+        if shape:
+            c.set_launch(*shape)
+        out.append(step(1))
+    (a, ia), (b, ib) = out
+    assert a["retries"] == 1 and b["retries"] == 0 and b["wave_launches"] == 0
+    assert np.array_equal(ia, ib) and a["rays"] == b["rays"]
