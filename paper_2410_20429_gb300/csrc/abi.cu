@@ -585,9 +585,9 @@ mars_status cache_create_impl(const mars_scene* s, const mars_cache_desc* d, cud
     return cleanup(e, "counter alloc");
   if (!(d->techniques & MARS_TECH_LIGHT)) {
     c->tail_blocks = s->num_sms * tail_occupancy();
-    if ((e = dev_alloc((void**)&c->d_tail_rounds, sizeof(uint4) * c->lanes * c->tail_blocks * (TAIL_ROUNDS + 1), st)) !=
-        cudaSuccess)
-      return cleanup(e, "counter alloc");
+    const size_t rounds = sizeof(uint4) * c->lanes * c->tail_blocks * (TAIL_ROUNDS + 1);
+    if ((e = dev_alloc((void**)&c->d_tail_rounds, rounds, st)) != cudaSuccess) return cleanup(e, "counter alloc");
+    c->device_bytes = rounds;
   }
   c->h_ctr = (DevCounters*)pinned_acquire(sizeof(DevCounters));
   if (!c->h_ctr) return cleanup(cudaErrorMemoryAllocation, "pinned alloc");
@@ -700,7 +700,7 @@ mars_status cache_create_impl(const mars_scene* s, const mars_cache_desc* d, cud
     c->dc.oct_cap_nodes = cap_nodes;
     c->dc.split_samples = d->split_samples > 0.0f ? d->split_samples : 4096.0f;
   }
-  c->device_bytes = cache_footprint(cells, pixels, d->max_depth, d->techniques, cap);
+  c->device_bytes += cache_footprint(cells, pixels, d->max_depth, d->techniques, cap);
   const bool light = (d->techniques & MARS_TECH_LIGHT) != 0;
   if ((e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking)) != cudaSuccess)
     return cleanup(e, "side stream");

@@ -344,3 +344,12 @@ def test_k_tail_keeps_to_the_room_a_launch_shape_leaves(mars, cap, threads, bloc
     (a, ia), (b, ib) = out
     assert a["retries"] == 1 and b["retries"] == 0 and b["wave_launches"] == 0
     assert np.array_equal(ia, ib) and a["rays"] == b["rays"]
+
+
+def test_device_bytes_count_the_rounds_of_k_tail(mars):
+    """A buffer of rounds (16 bytes each, 96 and one more a block) for every lane of a
+    cache that may use k_tail."""
+    scene = mars.Scene(W.guided_room_scene(2, 64, 64, n_spheres=24))
+    for tech, has in ((TECH3, True), (W.TECH_BSDF | W.TECH_NEE | W.TECH_LIGHT, False)):
+        one, two = (mars.Cache(scene, 6, tech, 5, lanes=n).info()["device_bytes"] for n in (1, 2))
+        assert (two - one) % (16 * 97) == 0 and (two > one) == has
