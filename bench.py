@@ -6,7 +6,7 @@ four small ceiling lights), max depth 10, techniques BSDF + NEE + guided,
 pixel rendered with the MARS counts, the image statistics, and the count /
 guide update.  The first W steps are the warm-up iterations (beta = 1).
 
-Printed (one JSON line, rank 0):
+Printed (one JSON line, rank 0; its long sections in full in the file --details):
   value      path vertices per second (closest-hit queries) over the K timed
              steps, device time from CUDA events on the rendering stream
   e2e        the same metric through the C ABI with the image returned to pinned
@@ -285,6 +285,19 @@ def reduce_over_ranks(total_ms, units, world, device):
     return float(t.item()), float(v.item())
 
 
+def short_line(line, details):
+    """The line as printed: sections of more than 500 characters by their plain values,
+    numbers and short texts, so that whoever keeps the last few kilobytes of a
+    program's output has all of it; the whole one is in the file `details`."""
+    out = {}
+    for k, v in line.items():
+        if isinstance(v, dict) and len(json.dumps(v)) > 500 and k not in ("config", "clocks"):
+            v = {q: w for q, w in v.items() if not isinstance(w, (dict, list)) and len(json.dumps(w)) <= 60}
+        if v != {}:
+            out[k] = v
+    return {**out, "details": details}
+
+
 def run_mars(args):
     import torch
     import paper_2410_20429_gb300 as M
@@ -556,7 +569,9 @@ def run_mars(args):
     if world > 1:
         dist.barrier()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        with open(args.details, "w") as f:
+            json.dump(line, f, indent=1)
+        print(json.dumps(short_line(line, args.details)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 
@@ -1253,6 +1268,7 @@ def main():
                     "block, blocks per SM and register cap of trace, shade, shadow, reverse); skips the autotuner")
     ap.add_argument("--clocks-csv", default="", help="where the nvidia-smi samples of the timed region go "
                     "('{rank}' is replaced by the rank; default: the temp directory)")
+    ap.add_argument("--details", default="bench_details.json", help="file for the whole line, every section in full")
     ap.add_argument("--arena-capacity", type=int, default=0, help="queue arena slots (0 = library default)")
     args = ap.parse_args()
     if args.warmup < 3 and args.impl == "mars":

@@ -1,6 +1,7 @@
 """CPU checks of the benchmark's measurement helpers: the clock-sample summary
 (window filtering, throttle reasons), relMSE and the single-rank aggregation."""
 import datetime
+import json
 import time
 
 import numpy as np
@@ -144,3 +145,21 @@ def test_measured_traffic_is_per_unit_and_keyed_by_the_sources(tmp_path, monkeyp
     assert all(10.0 < v < 1000.0 for v in vals.values())
     monkeypatch.setattr(bench, "kernel_sources_sha", lambda: "0" * 64)
     assert bench.measured_traffic() == {}
+
+
+def test_the_printed_line_is_short_and_keeps_the_measured_figures():
+    """Sections in full make some 20 kilobytes; printed are a few, with every plain value."""
+    per = {f"k{i}": {"achieved": float(i), "note": "x" * 200} for i in range(20)}
+    line = {"metric": bench.METRIC, "value": 1.0, "unit": bench.UNIT, "ms_per_step": 2.0,
+            "config": {"workload": "w", "l2": "y" * 600}, "clocks": {"sm_mhz": 2070.0, "reasons": [], "window": "z" * 500},
+            "e2e": {"value": 3.0, "unit": bench.UNIT, "h2d_bytes_per_step": 48, "d2h_bytes_per_step": 9,
+                    "iterations": "r" * 600, "graph_captures": {"a": 0}},
+            "roofline": {"kernel": "k_trace", "frac": 0.5, "traffic": None, "kernels": per},
+            "large_scene": per, "efficiency": {"ratio": 1.1, **per}, "convergence": {"mean_beta": [[0.1] * 3] * 200}}
+    s = bench.short_line(line, "d.json")
+    assert len(json.dumps(s)) < 4000 and s["details"] == "d.json"
+    for k in ("metric", "value", "unit", "ms_per_step", "config", "clocks"):
+        assert s[k] == line[k]
+    assert s["e2e"] == {k: line["e2e"][k] for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")}
+    assert s["roofline"] == {"kernel": "k_trace", "frac": 0.5, "traffic": None} and s["efficiency"] == {"ratio": 1.1}
+    assert "large_scene" not in s and "convergence" not in s
