@@ -842,32 +842,32 @@ static DevCache lane_cache(const mars_cache* c, int l) {
 // The depth from which on an iteration of `pixels` pixels a lane, with a ray arena
 // of `cap` slots a lane, runs in k_tail (with light connections: joins its waves'
 // side kernels, which needs no room); 0: nowhere.  The first wave of at most
-// kTailRays rays over the lanes, its size and those of the deeper waves taken from the last
-// iteration's rays per pixel (the first wave's is known), if what the waves
-// before leave of the arena holds the rest with tail_margin to spare -- a block's
-// subtrees may be larger than the average -- and, from the first wave on, 1.5 rays
-// per pixel and depth (a job's first iterations have little or no history).  The
-// NEE samples must fit as well, taken as spread over the waves like their rays.
+// kTailRays rays a lane -- with two lanes, whose kernels fill each other's gaps, also
+// of at most kTailMean rays a depth from it on, both lanes together --, its size and
+// those of the deeper waves taken from the last iteration's rays per pixel (the
+// first wave's is known), if what the waves before leave of the arena holds the rest
+// with tail_margin to spare -- a block's subtrees may be larger than the average --
+// and, from the first wave on, 1.5 rays per pixel and depth (a job's first
+// iterations have little or no history).  The NEE samples must fit as well, taken as
+// spread over the waves like their rays.
 // tail_margin doubles when slices overflow and comes back down by half in 64
 // iterations without one, so that a job whose subtrees stay uneven pays for a
 // failed attempt once in that many and one whose counts settle gets its tail back.
-// kTailRays: at 30 000, 60 000, 120 000 and 250 000 the 512^2 room's warm-up took
-// 0.833, 0.819, 0.821 and 0.875 ms, its iterations with learned counts 1.159, 1.153,
-// 1.177 and 1.340, the heightfield at 1024^2 2.44, 2.40, 2.46 and 2.51; without
-// k_tail 0.844, 1.165 and 2.63.  Larger waves fill the GPU by themselves, and the
-// waves of two lanes fill it together: with 65536 rays a lane, twice that in all,
-// the 512^2 room with counts learned over 20 iterations rendered 1610 to 1652
-// Mvertices/s in two lanes, with 32768 a lane 1715 to 1719 and without k_tail 1705 to
-// 1725 (in one lane all three 1616 to 1644); a drawn room's learned-count iteration
-// 1.35 -> 1.26 ms, the heightfield at 1024^2 2.27 -> 2.23.
-constexpr double kTailRays = 65536.0;
-// A depth in use is kept while its wave stays below kTailBand times that and no
-// earlier wave falls as far below it: next to the best depth the time changes by 1
-// or 2 %, and another depth is another recording of the iteration's graph.
-constexpr double kTailBand = 1.5;
+// Larger waves fill the GPU by themselves.  Iterations in two lanes, ms, without
+// k_tail and with it from each depth (its rays a depth in thousands):
+//   512^2 room, warm-up          0.839  from 5 (52) 0.819, 6 (42) 0.816, 7 (35) 0.829, 9 (24) 0.840
+//   512^2 room, given counts     1.157  from 5 (73) 1.170, 6 (52) 1.141, 7 (38) 1.143, 9 (21) 1.155
+//   512^2 room, learned counts   1.467  from 6 (69) 1.531, 7 (51) 1.532, 8 (38) 1.450, 9 (30) 1.467
+//   524k triangles, 283 x 1385   1.198  from 3 (68) 1.300, 4 (30) 1.171, 5 (16) 1.185
+//   131k triangles, 1024^2       2.64   from 5 (20) 2.42, 6 (8) 2.44
+constexpr double kTailRays = 65536.0, kTailMean = 49152.0;
+// A depth in use is kept while its waves stay below kTailBand times that and no
+// earlier depth's fall as far below it: next to the best depth the time changes by 1
+// to 5 %, and another depth is another recording of the iteration's graph.  The waves
+// of a steady job's iterations differ by some 3 %.
+constexpr double kTailBand = 1.1;
 constexpr double kTailMargin = 2.0, kTailMarginMost = 1 << 20;
 static int tail_depth(const mars_cache* c, int64_t pixels, uint64_t cap, int lanes) {
-  const double most = kTailRays / lanes;
   const bool light = (c->techniques & MARS_TECH_LIGHT) != 0;
   if (!light && (c->tail_blocks <= 0 || cap > (1ull << 31))) return 0;
   const double scale = c->last_pixels > 0 ? (double)pixels / (double)c->last_pixels : 0.0;
@@ -875,7 +875,7 @@ static int tail_depth(const mars_cache* c, int64_t pixels, uint64_t cap, int lan
   for (int d = 1; d <= c->max_depth; ++d) after += scale * (double)c->last_wave[d];
   const double shadow = after > 0.0 ? scale * (double)c->last_shadow / after : 0.0;  // NEE samples a ray
   int rule = 0;       // the rule's depth
-  double at = 0.0;    // and its wave
+  double at = 0.0;    // its waves over what the rule allows
   bool stay = false;  // the last iteration's depth still serves
   for (int k = 1; k <= c->max_depth && (k == 1 || c->last_pixels > 0); ++k) {
     const double wave = k == 1 ? (double)pixels : scale * (double)c->last_wave[k];
@@ -884,10 +884,13 @@ static int tail_depth(const mars_cache* c, int64_t pixels, uint64_t cap, int lan
     after -= scale * (double)c->last_wave[k];
     const double least = k == 1 ? 1.5 * (c->max_depth - 1) * (double)pixels : 0.0;
     if (!light && !(shadow_fits && (double)cap - before >= std::max(c->tail_margin * after, least))) continue;
-    if (rule == 0 && wave <= most) rule = k, at = wave;
-    if (k > 1 && k == c->last_tail && wave <= kTailBand * most) stay = true;
+    double load = wave / kTailRays;
+    if (lanes > 1)
+      load = std::max(load, lanes * (wave + std::max(after, least)) / (c->max_depth - k + 1) / kTailMean);
+    if (rule == 0 && load <= 1.0) rule = k, at = load;
+    if (k > 1 && k == c->last_tail && load <= kTailBand) stay = true;
   }
-  if (stay && rule != c->last_tail && (rule == 0 || rule > c->last_tail || kTailBand * at > most))
+  if (stay && rule != c->last_tail && (rule == 0 || rule > c->last_tail || kTailBand * at > 1.0))
     return c->last_tail;
   return rule;
 }
