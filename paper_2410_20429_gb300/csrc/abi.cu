@@ -1130,13 +1130,17 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
       // The last few are kept: a job that goes back and forth between tail depths,
       // modes or image buffers records each once.  The iteration that finds none is
       // launched directly, and its graph recorded while the GPU works on it: a
-      // recording takes the host about a quarter of a 512^2 iteration's time.
+      // recording takes the host about a quarter of a 512^2 iteration's time.  Where
+      // k_tail renders whole path trees it has a handful of kernels and is recorded
+      // sooner than they are launched one by one (first iteration of the 64^2 box 166 and
+      // 159 us, of the 128^2 room 540 and 529).
+      const bool few = tail == 1 && !(c->techniques & MARS_TECH_LIGHT);
       auto found = std::find_if(c->graphs.begin(), c->graphs.end(), [&](const auto& g) { return g.key == key; });
       if (found != c->graphs.end()) {
         std::rotate(c->graphs.begin(), found, found + 1);
         if ((e = cudaGraphLaunch(c->graphs.front().exec, st)) != cudaSuccess) return poison(c, e, "graph launch");
       } else {
-        if ((e = enqueue(st)) != cudaSuccess) return poison(c, e, "render launch");
+        if (!few && (e = enqueue(st)) != cudaSuccess) return poison(c, e, "render launch");
         NvtxRange nvtx_capture("mars:graph_capture");
         cudaGraph_t graph = nullptr;
         if ((e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
@@ -1157,6 +1161,7 @@ mars_status render_iteration_impl(mars_cache* c, const mars_iter_params* p, floa
         }
         c->graphs.insert(c->graphs.begin(), {key, exec});
         c->graph_captures += 1;
+        if (few && (e = cudaGraphLaunch(exec, st)) != cudaSuccess) return poison(c, e, "graph launch");
       }
     } else if ((e = enqueue(st)) != cudaSuccess) {
       return poison(c, e, "render launch");
