@@ -54,7 +54,7 @@ VERT_GUIDE_BYTES = 16   # V4 for a traced ray when the guided technique learns
 SAMPLE_BYTES = 16       # S: one float4 per slot
 EST_READ_BYTES = 16     # pixel estimate read per estimator vertex
 SHADOW_VALUE_BYTES = 16  # SH2 per NEE sample
-SHADOW_RAY_BYTES = 36   # SH0, SH1 and the work-list entry per traced shadow ray
+SHADOW_RAY_BYTES = 32   # SH0, SH1 per traced shadow ray
 SLOT_BYTES = RAY_BYTES + HIT_BYTES + V0_BYTES + VERT_EST_BYTES + VERT_GUIDE_BYTES + SAMPLE_BYTES
 
 
@@ -1251,7 +1251,7 @@ def main():
     ap.add_argument("--ref-pixels-per-step", type=int, default=65536)
     ap.add_argument("--no-autotune", action="store_true")
     ap.add_argument("--bvh", default="sah", choices=sorted(BVH_KINDS),
-                    help="hierarchy of the closest-hit and shadow queries (results do not depend on it)")
+                    help="hierarchy that the rays walk")
     ap.add_argument("--no-graphs", action="store_true", help="launch every kernel directly (no CUDA graph replay)")
     ap.add_argument("--lanes", type=int, default=2, choices=[1, 2],
                     help="concurrent pixel-tile lanes the cache is created with (the autotuner keeps one or all)")

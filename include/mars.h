@@ -91,7 +91,7 @@ typedef enum { MARS_WEIGHTS_AWARE = 0, MARS_WEIGHTS_UNAWARE = 1 } mars_weights;
  * camera: pinhole origin, look-at point, up vector, vertical FOV in degrees;
  *   width x height pixels, one box-filtered sample per pixel per iteration.
  * bvh: the hierarchy the closest-hit and shadow queries traverse (results do
- *   not depend on it): MARS_BVH_SAH (0) a top-down build on the host with the
+ *   not depend on it, see mars_scene_create): MARS_BVH_SAH (0) a top-down build on the host with the
  *   surface-area heuristic; MARS_BVH_LBVH a linear BVH built on the device
  *   (Morton codes, Karras hierarchy).  reserved: 0. */
 #define MARS_BVH_SAH 0
@@ -324,7 +324,9 @@ typedef struct {
  * bottom-up bounds); either is validated on the host and collapsed into the
  * 4-wide hierarchy that every ray walks -- and the light-selection table
  * (probability proportional to area x mean radiance).  Results do not depend
- * on the hierarchy.  Synchronises `stream` before returning.  Errors: INVALID_ARG (no primitives, bad sizes,
+ * on the hierarchy, but for rays that meet two primitives, one of them a sphere, at
+ * distances within the rounding of the sphere's (some 3 in 10^8 rays among thousands
+ * of spheres).  Synchronises `stream` before returning.  Errors: INVALID_ARG (no primitives, bad sizes,
  * material index out of range, emitting sphere/triangle), OOM, CUDA. */
 mars_status mars_scene_create(const mars_scene_desc* desc, void* stream, mars_scene** out);
 mars_status mars_scene_destroy(mars_scene* scene);

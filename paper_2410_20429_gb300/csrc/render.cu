@@ -248,9 +248,9 @@ size_t shade_smem(int threads) { return (size_t)(threads / 32) * sizeof(ShadeWar
 // starts with, is the 64, 80 and 64 register one for trace, shade and shadow:
 // uncapped they take 88, 144 and 77, and the kernels, which wait on loads most of
 // the time, lose more to the warps that then do not fit than they gain
-// (iterations with the caps against without: guided room 512^2 0.94 -> 0.89 ms
-// in the warm-up and 1.44 -> 1.25 with learned counts, 131k triangles at 1024^2
-// 3.62 -> 2.97, 524k at 2048^2 13.4 -> 11.7).  k_reverse keeps its registers
+// (iterations with the caps against without, both before the pools of rays: guided
+// room 512^2 0.94 -> 0.89 ms in the warm-up and 1.44 -> 1.25 with given counts, 131k
+// triangles at 1024^2 3.62 -> 2.97, 524k at 2048^2 13.4 -> 11.7).  k_reverse keeps its registers
 // (capped at 80, 512^2 warm-up 0.86 -> 0.91 ms).
 using TraceFn = void (*)(const DevScene, const DevCache, const Arena, const IterArgs*, const int);
 using ShadowFn = void (*)(const DevScene, const DevCache, const Arena, const int, const int);

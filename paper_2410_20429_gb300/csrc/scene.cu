@@ -201,7 +201,7 @@ cudaError_t build_bvh(const float4* d_box, int n, const float lo[3], const float
 // the same node format; siblings get adjacent node numbers.  A range that
 // could otherwise end deeper than kMaxDepth levels is split at its centroid
 // median along the widest axis from there on, so no leaf lies deeper than
-// kMaxDepth and the traversal stacks (48 entries) never overflow.
+// kMaxDepth (collapse_bvh4 checks the stack entries that a traversal needs).
 namespace {
 struct HBox {
   float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};

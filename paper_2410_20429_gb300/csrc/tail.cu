@@ -15,11 +15,11 @@
 // fused multiply-adds there spelled out, so that an image does not depend on
 // which of the two rendered it.
 // Bound by latency: the chain of the slowest ray of each round.  Measured per
-// iteration, wave kernels alone -> with the tail: 64^2 box 0.150 -> 0.121 ms,
-// 128^2 room of 459 spheres 0.573 -> 0.482, 317 x 203 room 0.536 -> 0.510, 128^2 and
-// 256^2 heightfield of 131k triangles 0.72 -> 0.38 and 0.95 -> 0.58, 524k triangles
-// at 256^2 1.38 -> 0.92; from a deeper wave on 512^2 room 0.84 -> 0.82, heightfield
-// at 1024^2 2.63 -> 2.41.
+// iteration, wave kernels alone -> with the tail: 64^2 box 0.150 -> 0.123 ms,
+// 128^2 room of 459 spheres 0.575 -> 0.482, 317 x 203 room 0.532 -> 0.519, 128^2 and
+// 256^2 heightfield of 131k triangles 0.75 -> 0.39 and 0.96 -> 0.59, 524k triangles
+// at 256^2 1.38 -> 0.93; from a deeper wave on 512^2 room's warm-up 0.847 -> 0.824, with
+// given counts 1.170 -> 1.159, heightfield at 1024^2 2.65 -> 2.43.
 #define MARS_PIN_FMA
 #include "wave.cuh"
 
