@@ -285,17 +285,23 @@ def reduce_over_ranks(total_ms, units, world, device):
     return float(t.item()), float(v.item())
 
 
+# what the printed line keeps of its long sections
+_SCENE = ("ms_per_step", "mvertices_s")
+_EFFICIENCY = ("ratio", "ratio_scaled", "ratio_vs_own_guide")
+PRINTED = {"roofline": ("kernel", "bound", "achieved", "peak", "unit", "frac", "traffic"),
+           "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"),
+           "large_scene": _SCENE, "largest_scene": _SCENE, "precision": ("images_equal",),
+           "serving": ("failed", "iter_ms_p50", "iter_ms_p99", "job_s_p50", "job_s_p99", "throughput_mvertices_s"),
+           "efficiency": _EFFICIENCY, "efficiency_box": _EFFICIENCY, "efficiency_box_16": _EFFICIENCY,
+           "cpu_baseline": ("value", "unit", "cores", "kind", "sample"), "convergence": ()}
+
+
 def short_line(line, details):
-    """The line as printed: sections of more than 500 characters by their plain values,
-    numbers and short texts, so that whoever keeps the last few kilobytes of a
-    program's output has all of it; the whole one is in the file `details`."""
-    out = {}
-    for k, v in line.items():
-        if isinstance(v, dict) and len(json.dumps(v)) > 500 and k not in ("config", "clocks"):
-            v = {q: w for q, w in v.items() if not isinstance(w, (dict, list)) and len(json.dumps(w)) <= 60}
-        if v != {}:
-            out[k] = v
-    return {**out, "details": details}
+    """The line as printed: of the long sections what PRINTED names, so that whoever
+    keeps the last three kilobytes of a program's output has all of it; the whole
+    line is in the file `details`."""
+    out = {k: {q: v[q] for q in PRINTED[k] if q in v} if k in PRINTED else v for k, v in line.items()}
+    return {**{k: v for k, v in out.items() if v != {}}, "details": details}
 
 
 def run_mars(args):

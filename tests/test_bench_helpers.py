@@ -148,18 +148,26 @@ def test_measured_traffic_is_per_unit_and_keyed_by_the_sources(tmp_path, monkeyp
 
 
 def test_the_printed_line_is_short_and_keeps_the_measured_figures():
-    """Sections in full make some 20 kilobytes; printed are a few, with every plain value."""
+    """Sections in full make some 20 kilobytes; three are printed."""
     per = {f"k{i}": {"achieved": float(i), "note": "x" * 200} for i in range(20)}
-    line = {"metric": bench.METRIC, "value": 1.0, "unit": bench.UNIT, "ms_per_step": 2.0,
-            "config": {"workload": "w", "l2": "y" * 600}, "clocks": {"sm_mhz": 2070.0, "reasons": [], "window": "z" * 500},
-            "e2e": {"value": 3.0, "unit": bench.UNIT, "h2d_bytes_per_step": 48, "d2h_bytes_per_step": 9,
+    num = 1234.56789012345678
+    eff = {"ratio": num, "ratio_scaled": num, "ratio_vs_own_guide": num, "note": "n" * 900, **per}
+    line = {"metric": bench.METRIC, "value": num, "unit": bench.UNIT, "ms_per_step": num, "gpu_launches": 772,
+            "config": {"workload": "w" * 50, "l2": "y" * 60, "parallelism": "replicas x1", "rest": "z" * 120},
+            "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": [], "window": "z" * 60},
+            "e2e": {"value": num, "unit": bench.UNIT, "h2d_bytes_per_step": 48, "d2h_bytes_per_step": 3146240,
                     "iterations": "r" * 600, "graph_captures": {"a": 0}},
-            "roofline": {"kernel": "k_trace", "frac": 0.5, "traffic": None, "kernels": per},
-            "large_scene": per, "efficiency": {"ratio": 1.1, **per}, "convergence": {"mean_beta": [[0.1] * 3] * 200}}
-    s = bench.short_line(line, "d.json")
-    assert len(json.dumps(s)) < 4000 and s["details"] == "d.json"
-    for k in ("metric", "value", "unit", "ms_per_step", "config", "clocks"):
+            "roofline": {"kernel": "k_trace", "bound": "alu", "achieved": num, "peak": num, "unit": "TFLOP/s",
+                         "frac": 0.5, "traffic": None, "kernels": per},
+            "large_scene": {"ms_per_step": num, "mvertices_s": num, **per}, "largest_scene": {"ms_per_step": num, **per},
+            "serving": {"failed": 0, "iter_ms_p50": num, "iter_ms_p99": num, "efficiency": per},
+            "efficiency": eff, "efficiency_box": eff, "efficiency_box_16": eff, "precision": {"images_equal": True, **per},
+            "cpu_baseline": {"value": num, "unit": bench.UNIT, "cores": 16, "kind": "oracle", "sample": "s" * 180, **per},
+            "convergence": {"mean_beta": [[0.1] * 3] * 200}}
+    s = bench.short_line(line, "bench_details.json")
+    assert len(json.dumps(s)) < 2900 and s["details"] == "bench_details.json"
+    for k in ("metric", "value", "unit", "ms_per_step", "gpu_launches", "config", "clocks"):
         assert s[k] == line[k]
     assert s["e2e"] == {k: line["e2e"][k] for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")}
-    assert s["roofline"] == {"kernel": "k_trace", "frac": 0.5, "traffic": None} and s["efficiency"] == {"ratio": 1.1}
-    assert "large_scene" not in s and "convergence" not in s
+    assert s["roofline"]["frac"] == 0.5 and s["roofline"]["traffic"] is None and "kernels" not in s["roofline"]
+    assert s["efficiency"]["ratio"] == num and s["cpu_baseline"]["cores"] == 16 and "convergence" not in s
